@@ -19,8 +19,8 @@
 // into the cache at L_b .. L_b + n_causal - 1 by the warp that brings the
 // block tile in.
 //
-// The fp32 variant (attn_f32_kernel) is a plain SIMT kernel with fp32 FMAs
-// throughout, used for fp32 inputs.
+// The fp32 variant (attn_f32_kernel) runs on fp32 FMAs throughout, split over
+// key ranges with the same in-cluster merge.
 #include <math.h>
 
 #include "sbd_internal.cuh"
@@ -123,84 +123,362 @@ attn_combine_kernel(const float* __restrict__ part_o, const float* __restrict__ 
 }
 
 // ------------------------------------------------------------ fp32 variant
-// One CTA per (query row i, query head, sequence); keys in chunks of 128
-// with an online softmax; every product and sum in fp32 FMAs.
-__global__ void __launch_bounds__(128)
-attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ kc,
-                const float* __restrict__ vc, const int32_t* __restrict__ lens,
-                const float* __restrict__ kb, const float* __restrict__ vb,
-                float* __restrict__ out, int* err, int k, int Hq, int Hkv, int D, int Lmax,
-                float scale_log2, int n_causal, float* __restrict__ kc_app,
-                float* __restrict__ vc_app) {
-  __shared__ float qs[128];
-  __shared__ float ps[128];
-  __shared__ float red[4];
+// Split-KV attention on fp32 FMAs.  One CTA per (key range, KV head,
+// sequence, chunk of W RW packed rows r = i*G + g): keys pass through shared
+// memory in tiles of 64, each K/V element read from global memory once per
+// row chunk.  A warp owns RW rows in both products, so the softmax and P stay
+// inside the warp:
+//   S   lane = keys (lane, lane + 32) of the tile; Q rows are broadcast
+//       reads; even and odd dimensions add up in the two halves of packed
+//       fp32 FMAs (fma.rn.f32x2: two IEEE FMAs);
+//   P   through shared memory within the warp;
+//   O   lane = D / 32 consecutive dimensions; P values are broadcast reads.
+// The key ranges of a (sequence, KV head, chunk) are the CTAs of one
+// thread-block cluster and merge through distributed shared memory, so no
+// workspace is needed.
+// Bound: the FMAs of a full tile are 2 us of an SM (32 rows x 64 keys x 128
+// dimensions, twice); a tile measured 5.2 us with one CTA on the SM, the rest
+// being latencies between the phases that a second CTA covers in part.  With
+// 4 warps of 8 rows in place of 8 of 4: 30.3 against 28.6 us at the shape below.
+// The form before (one CTA per query row and head, each walking all keys,
+// uncoalesced) took 717 us at B = 2, k = 8, 32/8 heads of 128, 511-2048
+// cached keys, and 37 us at 4/2 heads of 64, k = 4, 128 keys (the smallest
+// configuration); this one takes 28.6 and 4.6 us (graph replays; the FMAs of
+// the first are 4.2 us of the whole chip, its bytes 3.1 us of HBM).
+constexpr int kF32Keys = 64;                 // keys per tile
+constexpr int kF32Granule = 16;              // key ranges are multiples of this
+
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(d)
+      : "l"(*reinterpret_cast<const unsigned long long*>(&a)),
+        "l"(*reinterpret_cast<const unsigned long long*>(&b)),
+        "l"(*reinterpret_cast<const unsigned long long*>(&c)));
+  return *reinterpret_cast<float2*>(&d);
+}
+__device__ __forceinline__ float2 lo2(const float4& v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(const float4& v) { return make_float2(v.z, v.w); }
+
+// 16 bytes global -> shared, asynchronously; zeros when !valid (src is not read).
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+               "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A float at this CTA's shared location `p`, read in CTA `rank` of the cluster.
+__device__ __forceinline__ float ld_rank(const float* p, int rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_rank2(const float* p, int rank) {
+  uint32_t a;
+  float2 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+
+struct F32Args {
+  const float *q, *kc, *vc;
+  const int32_t* lens;
+  const float *kb, *vb;
+  float* out;
+  int* err;
+  float *kc_app, *vc_app;      // writable caches for the causal rows, or NULL
+  int k, Hq, Hkv, G, M, Lmax, n_causal, splits, chunks;
+  float scale_log2;
+};
+
+template <int D>
+__host__ __device__ constexpr int f32_k_stride() { return D + 4; }   // lanes' rows in distinct banks
+
+template <int D, int RW, int W>
+constexpr size_t f32_smem_bytes() {
+  return sizeof(float) * ((size_t)W * RW * D                            // Q
+                          + (size_t)kF32Keys * (f32_k_stride<D>() + D)  // K, V tile
+                          + (size_t)W * RW * kF32Keys                   // P
+                          + 2 * W * RW);                                // m, l of the merge
+}
+
+template <int D, int RW, int W>
+__global__ void __launch_bounds__(32 * W)
+attn_f32_kernel(const F32Args a) {
+  constexpr int kF32Warps = W, kF32Threads = 32 * W;
+  constexpr int kRowsCta = kF32Warps * RW;
+  constexpr int kKS = f32_k_stride<D>();
+  constexpr int kPer = D / 32;                 // output dimensions per lane
+  constexpr int kC4 = D / 4;                   // 16-byte chunks of a row
+  extern __shared__ __align__(16) float sm[];
+  float* q_s = sm;                             // [kRowsCta][D]
+  float* k_s = q_s + kRowsCta * D;             // [kF32Keys][kKS]
+  float* v_s = k_s + kF32Keys * kKS;           // [kF32Keys][D]
+  float* p_s = v_s + kF32Keys * D;             // [kRowsCta][kF32Keys]
+  float* st_s = p_s + kRowsCta * kF32Keys;     // m, then l: [kRowsCta] each
+  float* o_s = k_s;                            // merge: [kRowsCta][D], over the dead K tile
+  static_assert(kRowsCta * D <= kF32Keys * kKS, "the partial rows fit the K tile");
+
   grid_dependency_wait();
-  const int i = blockIdx.x, hq = blockIdx.y, b = blockIdx.z;
-  const int G = Hq / Hkv, hkv = hq / G;
-  const int tid = threadIdx.x;
-  int len = lens[b];
-  if (len < 0 || len > Lmax) {
-    if (tid == 0) sbd_dev::record_error(err, SBD_DEVERR_CACHE_LEN);
-    len = len < 0 ? 0 : Lmax;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int split = blockIdx.x, hkv = blockIdx.y / a.chunks, chunk = blockIdx.y % a.chunks;
+  const int b = blockIdx.z;
+  int len = a.lens[b];
+  if (len < 0 || len > a.Lmax) {
+    if (tid == 0) record_error(a.err, SBD_DEVERR_CACHE_LEN);
+    len = len < 0 ? 0 : a.Lmax;
   }
-  const float* qrow = q + (((size_t)b * k + i) * Hq + hq) * D;
-  if (tid < D) qs[tid] = qrow[tid];
-  // The first CTA of each KV head writes a causal row's key and value into
-  // the cache; the attention below reads cache positions < len only.
-  if (kc_app && i < n_causal && hq % G == 0 && tid < D) {
-    if (len + n_causal <= Lmax) {
-      const size_t dst = (((size_t)b * Lmax + len + i) * Hkv + hkv) * D + tid;
-      const size_t src = (((size_t)b * k + i) * Hkv + hkv) * D + tid;
-      kc_app[dst] = kb[src];
-      vc_app[dst] = vb[src];
-    } else if (tid == 0 && i == 0) {
-      sbd_dev::record_error(err, SBD_DEVERR_CACHE_LEN);
+  const int total = len + a.k;
+  const int range = ((total + a.splits - 1) / a.splits + kF32Granule - 1) / kF32Granule * kF32Granule;
+  const int u_begin = min(total, split * range), u_end = min(total, u_begin + range);
+
+  // Cache and block rows are both Hkv * D floats apart; a thread always
+  // copies the same 16-byte column of a row.
+  const int row_floats = a.Hkv * D;
+  const int c_ld = 4 * (tid % kC4), j_ld = tid / kC4;
+  const size_t cache_off = ((size_t)b * a.Lmax * a.Hkv + hkv) * D + c_ld;
+  const size_t blk_off = ((size_t)b * a.k * a.Hkv + hkv) * D + c_ld;
+  auto load_tile = [&](float* dst, int stride, const float* cache, const float* blk, int t0) {
+    // rows up to the next multiple of 4 keys are zeros (PV takes 4 at a time)
+    const int n4 = (min(kF32Keys, u_end - t0) + 3) & ~3;
+#pragma unroll 4
+    for (int j = j_ld; j < n4; j += kF32Threads / kC4) {
+      const int u = t0 + j;
+      const bool valid = u < u_end;
+      const float* src = u < len ? cache + cache_off + (size_t)u * row_floats
+                                 : blk + blk_off + (size_t)(valid ? u - len : 0) * row_floats;
+      cp_async16(dst + j * stride + c_ld, src, valid);
+    }
+    cp_async_commit();
+  };
+  if (u_begin < u_end) load_tile(k_s, kKS, a.kc, a.kb, u_begin);
+
+  // Q rows of the chunk (zeros past M)
+  for (int e = tid; e < kRowsCta * kC4; e += kF32Threads) {
+    const int rl = e / kC4, c = e % kC4, r = chunk * kRowsCta + rl;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < a.M)
+      v = *reinterpret_cast<const float4*>(
+          a.q + (((size_t)b * a.k + r / a.G) * a.Hq + hkv * a.G + r % a.G) * D + 4 * c);
+    *reinterpret_cast<float4*>(q_s + rl * D + 4 * c) = v;
+  }
+  // The first CTA of each (sequence, KV head) writes the causal rows' keys
+  // and values into the cache; cache positions < len alone are read.
+  if (a.kc_app && split == 0 && chunk == 0) {
+    if (len + a.n_causal <= a.Lmax) {
+      for (int e = tid; e < a.n_causal * kC4; e += kF32Threads) {
+        const int i = e / kC4, c = e % kC4;
+        const size_t dst = (((size_t)b * a.Lmax + len + i) * a.Hkv + hkv) * D + 4 * c;
+        const size_t src = (((size_t)b * a.k + i) * a.Hkv + hkv) * D + 4 * c;
+        *reinterpret_cast<float4*>(a.kc_app + dst) = *reinterpret_cast<const float4*>(a.kb + src);
+        *reinterpret_cast<float4*>(a.vc_app + dst) = *reinterpret_cast<const float4*>(a.vb + src);
+      }
+    } else if (tid == 0) {
+      record_error(a.err, SBD_DEVERR_CACHE_LEN);
     }
   }
-  __syncthreads();
-  // causal rows of the block see the block keys j <= i only
-  const int total = len + (i < n_causal ? i + 1 : k);
-  float m = -INFINITY, l = 0.f, acc = 0.f;   // acc: output element d = tid
-  for (int c0 = 0; c0 < total; c0 += 128) {
-    const int u = c0 + tid;
-    float s = -INFINITY;
-    if (u < total) {
-      const float* key = (u < len) ? kc + (((size_t)b * Lmax + u) * Hkv + hkv) * D
-                                   : kb + (((size_t)b * k + (u - len)) * Hkv + hkv) * D;
-      float dot = 0.f;
-      for (int d = 0; d < D; ++d) dot = fmaf(qs[d], key[d], dot);
-      s = dot * scale_log2;
-    }
-    // block max
-    float mx = sbd_dev::warp_max(s);
-    if ((tid & 31) == 0) red[tid >> 5] = mx;
+
+  // this warp's rows: local rows RW*warp .. + RW - 1; keys u < vis[r] are seen
+  int vis[RW];
+#pragma unroll
+  for (int r = 0; r < RW; ++r) {
+    const int i = (chunk * kRowsCta + RW * warp + r) / a.G;
+    vis[r] = min(u_end, len + (i < a.n_causal ? i + 1 : a.k));
+  }
+  float m[RW], l[RW];                          // l: this lane's share of the row sum
+  float2 o[RW][kPer / 2];
+#pragma unroll
+  for (int r = 0; r < RW; ++r) {
+    m[r] = -INFINITY;
+    l[r] = 0.f;
+#pragma unroll
+    for (int c = 0; c < kPer / 2; ++c) o[r][c] = make_float2(0.f, 0.f);
+  }
+  const float* qw = q_s + RW * warp * D;
+  float* pw = p_s + RW * warp * kF32Keys;
+
+  for (int t0 = u_begin; t0 < u_end; t0 += kF32Keys) {
+    const int n = min(kF32Keys, u_end - t0);
+    load_tile(v_s, D, a.vc, a.vb, t0);
+    cp_async_wait<1>();                        // the K tile
     __syncthreads();
-    mx = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
-    __syncthreads();
-    const float mn = fmaxf(m, mx);
-    const float alpha = (m == -INFINITY) ? 0.f : exp2f(m - mn);
-    const float p = (s == -INFINITY) ? 0.f : exp2f(s - mn);
-    ps[tid] = p;
-    float psum = sbd_dev::warp_sum(p);
-    if ((tid & 31) == 0) red[tid >> 5] = psum;
-    __syncthreads();
-    psum = (red[0] + red[1]) + (red[2] + red[3]);
-    l = l * alpha + psum;
-    m = mn;
-    if (tid < D) {
-      acc *= alpha;
-      const int n = min(128, total - c0);
-      for (int j = 0; j < n; ++j) {
-        const int uu = c0 + j;
-        const float* val = (uu < len) ? vc + (((size_t)b * Lmax + uu) * Hkv + hkv) * D
-                                      : vb + (((size_t)b * k + (uu - len)) * Hkv + hkv) * D;
-        acc = fmaf(ps[j], val[tid], acc);
+    // ---- S: keys lane and lane + 32 of the tile
+    const bool two = n > 32;
+    float s[RW][2];
+    {
+      float2 acc[RW][2];
+#pragma unroll
+      for (int r = 0; r < RW; ++r) acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+      const float* k0 = k_s + lane * kKS;
+      const float* k1 = k0 + 32 * kKS;
+      if (two) {
+#pragma unroll 4
+        for (int c = 0; c < kC4; ++c) {
+          const float4 x0 = *reinterpret_cast<const float4*>(k0 + 4 * c);
+          const float4 x1 = *reinterpret_cast<const float4*>(k1 + 4 * c);
+#pragma unroll
+          for (int r = 0; r < RW; ++r) {
+            const float4 qv = *reinterpret_cast<const float4*>(qw + r * D + 4 * c);
+            acc[r][0] = ffma2(hi2(qv), hi2(x0), ffma2(lo2(qv), lo2(x0), acc[r][0]));
+            acc[r][1] = ffma2(hi2(qv), hi2(x1), ffma2(lo2(qv), lo2(x1), acc[r][1]));
+          }
+        }
+      } else {
+#pragma unroll 4
+        for (int c = 0; c < kC4; ++c) {
+          const float4 x0 = *reinterpret_cast<const float4*>(k0 + 4 * c);
+#pragma unroll
+          for (int r = 0; r < RW; ++r) {
+            const float4 qv = *reinterpret_cast<const float4*>(qw + r * D + 4 * c);
+            acc[r][0] = ffma2(hi2(qv), hi2(x0), ffma2(lo2(qv), lo2(x0), acc[r][0]));
+          }
+        }
+      }
+      // keys past the row's last visible one (their tile rows may hold
+      // anything) do not count
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        s[r][0] = t0 + lane < vis[r] ? (acc[r][0].x + acc[r][0].y) * a.scale_log2 : -INFINITY;
+        s[r][1] = two && t0 + lane + 32 < vis[r] ? (acc[r][1].x + acc[r][1].y) * a.scale_log2
+                                                 : -INFINITY;
       }
     }
-    __syncthreads();
+    // ---- softmax of the tile
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+      const float mn = fmaxf(m[r], warp_max(fmaxf(s[r][0], s[r][1])));
+      const float alpha = m[r] == -INFINITY ? 0.f : exp2f(m[r] - mn);
+      const float p0 = s[r][0] == -INFINITY ? 0.f : exp2f(s[r][0] - mn);
+      const float p1 = s[r][1] == -INFINITY ? 0.f : exp2f(s[r][1] - mn);
+      m[r] = mn;
+      l[r] = fmaf(l[r], alpha, p0 + p1);
+#pragma unroll
+      for (int c = 0; c < kPer / 2; ++c) {
+        o[r][c].x *= alpha;
+        o[r][c].y *= alpha;
+      }
+      pw[r * kF32Keys + lane] = p0;
+      pw[r * kF32Keys + lane + 32] = p1;
+    }
+    cp_async_wait<0>();                        // the V tile
+    __syncthreads();                           // every warp is done with the K tile, too
+    if (t0 + kF32Keys < u_end) load_tile(k_s, kKS, a.kc, a.kb, t0 + kF32Keys);
+    // ---- O += P V, 4 keys at a time
+#pragma unroll 2
+    for (int j = 0; j < n; j += 4) {
+      float2 v[4][kPer / 2];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if constexpr (kPer == 4) {
+          const float4 x = *reinterpret_cast<const float4*>(v_s + (j + e) * D + 4 * lane);
+          v[e][0] = lo2(x);
+          v[e][kPer / 2 - 1] = hi2(x);
+        } else {
+          v[e][0] = *reinterpret_cast<const float2*>(v_s + (j + e) * D + 2 * lane);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        const float4 p = *reinterpret_cast<const float4*>(pw + r * kF32Keys + j);
+#pragma unroll
+        for (int c = 0; c < kPer / 2; ++c) {
+          o[r][c] = ffma2(make_float2(p.x, p.x), v[0][c], o[r][c]);
+          o[r][c] = ffma2(make_float2(p.y, p.y), v[1][c], o[r][c]);
+          o[r][c] = ffma2(make_float2(p.z, p.z), v[2][c], o[r][c]);
+          o[r][c] = ffma2(make_float2(p.w, p.w), v[3][c], o[r][c]);
+        }
+      }
+    }
+    __syncthreads();                           // the V tile is consumed
   }
-  if (tid < D) out[(((size_t)b * k + i) * Hq + hq) * D + tid] = acc / l;
+  grid_dependents_launch();
+
+  auto store_row = [&](int rl, const float2 (&x)[kPer / 2], float inv_of) {
+    const int r = chunk * kRowsCta + rl;
+    if (r >= a.M) return;
+    float* dst = a.out + (((size_t)b * a.k + r / a.G) * a.Hq + hkv * a.G + r % a.G) * D + kPer * lane;
+#pragma unroll
+    for (int c = 0; c < kPer / 2; ++c)
+      *reinterpret_cast<float2*>(dst + 2 * c) = make_float2(x[c].x / inv_of, x[c].y / inv_of);
+  };
+  if (a.splits == 1) {
+#pragma unroll
+    for (int r = 0; r < RW; ++r) store_row(RW * warp + r, o[r], warp_sum(l[r]));
+    return;
+  }
+  // ---- merge over the cluster: every CTA leaves its rows' maximum, sum and
+  // unnormalised O in shared memory; CTA `split` merges rows split,
+  // split + splits, ...  The second barrier keeps shared memory alive until
+  // every CTA has read it.
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < RW; ++r) {
+    const int rl = RW * warp + r;
+    const float lr = warp_sum(l[r]);
+#pragma unroll
+    for (int c = 0; c < kPer / 2; ++c)
+      *reinterpret_cast<float2*>(o_s + rl * D + kPer * lane + 2 * c) = o[r][c];
+    if (lane == 0) {
+      st_s[rl] = m[r];
+      st_s[kRowsCta + rl] = lr;
+    }
+  }
+  cluster_sync_all();
+  for (int rl = split + a.splits * warp; rl < kRowsCta && chunk * kRowsCta + rl < a.M;
+       rl += a.splits * kF32Warps) {
+    const float ms = lane < a.splits ? ld_rank(st_s + rl, lane) : -INFINITY;
+    const float ls = lane < a.splits ? ld_rank(st_s + kRowsCta + rl, lane) : 0.f;
+    const float mx = warp_max(ms);
+    const float w = mx == -INFINITY ? (lane < a.splits ? 1.f : 0.f) : exp2f(ms - mx);
+    const float lsum = warp_sum(w * ls);
+    float2 acc[kPer / 2];
+#pragma unroll
+    for (int c = 0; c < kPer / 2; ++c) acc[c] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int e = 0; e < a.splits; ++e) {
+      const float we = __shfl_sync(0xffffffffu, w, e);
+#pragma unroll
+      for (int c = 0; c < kPer / 2; ++c) {
+        const float2 x = ld_rank2(o_s + rl * D + kPer * lane + 2 * c, e);
+        acc[c].x = fmaf(we, x.x, acc[c].x);
+        acc[c].y = fmaf(we, x.y, acc[c].y);
+      }
+    }
+    store_row(rl, acc, lsum);
+  }
+  cluster_sync_all();
+}
+
+// The instance for M packed rows: few rows per warp at small M (a small block
+// keeps every warp busy), else chunks of 32 rows on 8 warps.
+struct F32Kernel {
+  const void* fn;
+  size_t smem;
+  int rows;          // packed rows per CTA
+  int threads;
+};
+F32Kernel f32_kernel_for(int D, int M) {
+  if (D == 128) {
+    if (M <= 8) return {(const void*)attn_f32_kernel<128, 2, 4>, f32_smem_bytes<128, 2, 4>(), 8, 128};
+    if (M <= 16) return {(const void*)attn_f32_kernel<128, 4, 4>, f32_smem_bytes<128, 4, 4>(), 16, 128};
+    return {(const void*)attn_f32_kernel<128, 4, 8>, f32_smem_bytes<128, 4, 8>(), 32, 256};
+  }
+  if (M <= 8) return {(const void*)attn_f32_kernel<64, 2, 4>, f32_smem_bytes<64, 2, 4>(), 8, 128};
+  if (M <= 16) return {(const void*)attn_f32_kernel<64, 4, 4>, f32_smem_bytes<64, 4, 4>(), 16, 128};
+  return {(const void*)attn_f32_kernel<64, 4, 8>, f32_smem_bytes<64, 4, 8>(), 32, 256};
 }
 
 }  // namespace
@@ -219,6 +497,24 @@ static int choose_splits(int pairs, int n_tiles_max, int sms) {
   return s < max_s ? s : max_s;
 }
 
+// Key ranges of the fp32 kernel per (sequence, KV head, row chunk): as many
+// as two CTAs per SM allow, one range per kF32Granule keys at most, in a
+// cluster size whose clusters the device holds all at once (a second wave
+// doubles the time: B = 2, k = 8, 2048 keys, 16 jobs, measured with the
+// 4-warp form 30.3 us at 12 ranges, 34.0 at 16, where 14 clusters fit).
+static int f32_splits(const AttnPlan& p) {
+  const F32Kernel kern = f32_kernel_for(p.D, p.M);
+  const long long jobs = (long long)p.B * p.Hkv * ((p.M + kern.rows - 1) / kern.rows);
+  const long long keys = (long long)p.Lmax + p.k;
+  const long long by_keys = (keys + kF32Granule - 1) / kF32Granule;
+  if (jobs <= 0) return 1;
+  for (int s : {16, 12, 10, 8, 6, 5, 4, 3, 2}) {
+    if (s > by_keys || s * jobs > 2ll * num_sms()) continue;
+    if (cluster_slots(kern.fn, kern.threads, kern.smem, s) >= jobs) return s;
+  }
+  return 1;
+}
+
 AttnPlan attn_plan(const sbd_attn_desc& d) {
   AttnPlan p;
   p.B = d.batch;
@@ -235,7 +531,7 @@ AttnPlan attn_plan(const sbd_attn_desc& d) {
   p.scale_log2 = scale * kLog2e;
   const int tiles = (p.Lmax + kTileKeys - 1) / kTileKeys + 1;
   if (!p.bf16) {
-    p.splits = 1;
+    p.splits = f32_splits(p);
   } else if (d.num_splits > 0) {
     p.splits = d.num_splits;
   } else {
@@ -249,7 +545,7 @@ AttnPlan attn_plan(const sbd_attn_desc& d) {
   // cached keys, 12 splits in clusters took 12.9 us against 13.9 us for 19
   // splits merged by attn_combine_kernel.  Otherwise the partials go through
   // the workspace and attn_combine_kernel.
-  p.cluster = false;
+  p.cluster = !p.bf16 && p.splits > 1;
   if (p.bf16 && p.B > 0 && p.splits >= 2) {
     const int hi = p.splits < 16 ? p.splits : 16;
     const int lo = d.num_splits > 0 ? p.splits : (3 * p.splits + 4) / 5;
@@ -280,20 +576,34 @@ sbd_status attn_launch(const AttnPlan& p, const void* q, const void* kc, const v
   if (p.B == 0) return SBD_OK;
   int* err = device_error_word();
   if (!p.bf16) {
-    const float *qf = (const float*)q, *kcf = (const float*)kc, *vcf = (const float*)vc;
-    const float *kbf = (const float*)kb, *vbf = (const float*)vb;
-    float* of = (float*)out;
-    int k = p.k, Hq = p.Hq, Hkv = p.Hkv, D = p.D, Lmax = p.Lmax;
-    float sl2 = p.scale_log2;
-    int nc = p.n_causal;
-    float* kca = (float*)kc_app;
-    float* vca = (float*)vc_app;
-    void* args[] = {(void*)&qf,  (void*)&kcf, (void*)&vcf,  (void*)&lens, (void*)&kbf,
-                    (void*)&vbf, (void*)&of,  (void*)&err,  (void*)&k,    (void*)&Hq,
-                    (void*)&Hkv, (void*)&D,   (void*)&Lmax, (void*)&sl2,  (void*)&nc,
-                    (void*)&kca, (void*)&vca};
-    return launch_pdl((const void*)attn_f32_kernel, dim3(p.k, p.Hq, p.B), dim3(128), 0, st, args,
-                      "attn_f32_kernel launch");
+    F32Args a;
+    a.q = (const float*)q;
+    a.kc = (const float*)kc;
+    a.vc = (const float*)vc;
+    a.lens = lens;
+    a.kb = (const float*)kb;
+    a.vb = (const float*)vb;
+    a.out = (float*)out;
+    a.err = err;
+    a.kc_app = (float*)kc_app;
+    a.vc_app = (float*)vc_app;
+    a.k = p.k;
+    a.Hq = p.Hq;
+    a.Hkv = p.Hkv;
+    a.G = p.G;
+    a.M = p.M;
+    a.Lmax = p.Lmax;
+    a.n_causal = p.n_causal;
+    a.splits = p.splits;
+    a.scale_log2 = p.scale_log2;
+    const F32Kernel kern = f32_kernel_for(p.D, p.M);
+    a.chunks = (p.M + kern.rows - 1) / kern.rows;
+    const cudaError_t e = cudaFuncSetAttribute(
+        kern.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kern.smem);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_f32_kernel)");
+    void* args[] = {(void*)&a};
+    return launch_pdl(kern.fn, dim3(p.splits, p.Hkv * a.chunks, p.B), dim3(kern.threads),
+                      kern.smem, st, args, "attn_f32_kernel launch", p.splits);
   }
 
   // 4-D tensor maps over the caches: dims (D, Hkv, Lmax, B), 64x64 boxes.

@@ -185,6 +185,34 @@ int max_active_clusters(const void* fn, dim3 grid, dim3 block, size_t smem, int 
   return n;
 }
 
+int cluster_slots(const void* fn, int threads, size_t smem, int cluster_x) {
+  struct Entry {
+    int dev;
+    const void* fn;
+    int cluster_x;
+    int clusters;
+  };
+  static std::mutex mu;
+  static Entry kept[64];
+  static int n_kept = 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    for (int i = 0; i < n_kept; ++i)
+      if (kept[i].dev == dev && kept[i].fn == fn && kept[i].cluster_x == cluster_x)
+        return kept[i].clusters;
+  }
+  const int clusters =
+      max_active_clusters(fn, dim3(cluster_x), dim3(threads), smem, cluster_x);
+  std::lock_guard<std::mutex> lock(mu);
+  if (n_kept < 64) kept[n_kept++] = Entry{dev, fn, cluster_x, clusters};
+  return clusters;
+}
+
 }  // namespace sbd
 
 using sbd::aligned16;

@@ -100,6 +100,9 @@ sbd_status launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem, cudaSt
 // memory each) the current device can hold at once; 0 when the shape cannot
 // be launched as clusters.
 int max_active_clusters(const void* fn, dim3 grid, dim3 block, size_t smem, int cluster_x);
+// The same for the current device, kept per (device, kernel, cluster size): for
+// the host path of a launch.
+int cluster_slots(const void* fn, int threads, size_t smem, int cluster_x);
 
 }  // namespace sbd
 

@@ -143,3 +143,19 @@ def test_bf16_random_shapes(sbd, case):
                    cache_len=(0, Lmax))
     _check(sbd, w, _inputs(w, case, lens), n_causal, num_splits=splits)
     assert sbd.sbd_device_error() == 0
+
+
+@pytest.mark.parametrize("n_causal", [0, 1, 3])
+@pytest.mark.parametrize("G,k,D", [(1, 3, 64), (2, 4, 128), (3, 3, 64), (4, 4, 64), (17, 3, 128), (4, 8, 128),
+                                   (3, 11, 64), (4, 32, 128), (33, 31, 64)])
+def test_f32_split_and_tile_edges(sbd, G, k, D, n_causal):
+    """fp32 kernel: packed rows around the row chunks (8, 16, 32) and far
+    above one, cache lengths around the 16-key granule and 64-key tile, and
+    rows whose keys all lie in other ranges."""
+    lens = [0, 1, 15, 16, 60, 61, 64, 65, 127, 200, 513]
+    w = gen.shrink(gen.get_workload("tiny_f32"), batch=len(lens), block_k=k, n_q_heads=G, n_kv_heads=1,
+                   head_dim=D, cache_len=(0, 513 + k))
+    _check(sbd, w, _inputs(w, G * k, lens), n_causal)
+    w = gen.shrink(w, batch=1, cache_len=(0, 2100))
+    _check(sbd, w, _inputs(w, G * k + 1, [2081]), n_causal)
+    assert sbd.sbd_device_error() == 0
