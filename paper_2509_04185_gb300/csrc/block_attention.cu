@@ -129,8 +129,7 @@ attn_combine_kernel(const float* __restrict__ part_o, const float* __restrict__ 
 // row chunk.  A warp owns RW rows in both products, so the softmax and P stay
 // inside the warp:
 //   S   lane = keys (lane, lane + 32) of the tile; Q rows are broadcast
-//       reads; even and odd dimensions add up in the two halves of packed
-//       fp32 FMAs (fma.rn.f32x2: two IEEE FMAs);
+//       reads;
 //   P   through shared memory within the warp;
 //   O   lane = D / 32 consecutive dimensions; P values are broadcast reads.
 // The key ranges of a (sequence, KV head, chunk) are the CTAs of one
@@ -148,31 +147,6 @@ attn_combine_kernel(const float* __restrict__ part_o, const float* __restrict__ 
 constexpr int kF32Keys = 64;                 // keys per tile
 constexpr int kF32Granule = 16;              // key ranges are multiples of this
 
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;"
-      : "=l"(d)
-      : "l"(*reinterpret_cast<const unsigned long long*>(&a)),
-        "l"(*reinterpret_cast<const unsigned long long*>(&b)),
-        "l"(*reinterpret_cast<const unsigned long long*>(&c)));
-  return *reinterpret_cast<float2*>(&d);
-}
-__device__ __forceinline__ float2 lo2(const float4& v) { return make_float2(v.x, v.y); }
-__device__ __forceinline__ float2 hi2(const float4& v) { return make_float2(v.z, v.w); }
-
-// 16 bytes global -> shared, asynchronously; zeros when !valid (src is not read).
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
-               "r"(valid ? 16 : 0)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -299,13 +273,13 @@ attn_f32_kernel(const F32Args a) {
     vis[r] = min(u_end, len + (i < a.n_causal ? i + 1 : a.k));
   }
   float m[RW], l[RW];                          // l: this lane's share of the row sum
-  float2 o[RW][kPer / 2];
+  float o[RW][kPer];
 #pragma unroll
   for (int r = 0; r < RW; ++r) {
     m[r] = -INFINITY;
     l[r] = 0.f;
 #pragma unroll
-    for (int c = 0; c < kPer / 2; ++c) o[r][c] = make_float2(0.f, 0.f);
+    for (int c = 0; c < kPer; ++c) o[r][c] = 0.f;
   }
   const float* qw = q_s + RW * warp * D;
   float* pw = p_s + RW * warp * kF32Keys;
@@ -319,9 +293,9 @@ attn_f32_kernel(const F32Args a) {
     const bool two = n > 32;
     float s[RW][2];
     {
-      float2 acc[RW][2];
+      float acc[RW][2];
 #pragma unroll
-      for (int r = 0; r < RW; ++r) acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+      for (int r = 0; r < RW; ++r) acc[r][0] = acc[r][1] = 0.f;
       const float* k0 = k_s + lane * kKS;
       const float* k1 = k0 + 32 * kKS;
       if (two) {
@@ -332,8 +306,8 @@ attn_f32_kernel(const F32Args a) {
 #pragma unroll
           for (int r = 0; r < RW; ++r) {
             const float4 qv = *reinterpret_cast<const float4*>(qw + r * D + 4 * c);
-            acc[r][0] = ffma2(hi2(qv), hi2(x0), ffma2(lo2(qv), lo2(x0), acc[r][0]));
-            acc[r][1] = ffma2(hi2(qv), hi2(x1), ffma2(lo2(qv), lo2(x1), acc[r][1]));
+            acc[r][0] = dot4(qv, x0, acc[r][0]);
+            acc[r][1] = dot4(qv, x1, acc[r][1]);
           }
         }
       } else {
@@ -341,19 +315,16 @@ attn_f32_kernel(const F32Args a) {
         for (int c = 0; c < kC4; ++c) {
           const float4 x0 = *reinterpret_cast<const float4*>(k0 + 4 * c);
 #pragma unroll
-          for (int r = 0; r < RW; ++r) {
-            const float4 qv = *reinterpret_cast<const float4*>(qw + r * D + 4 * c);
-            acc[r][0] = ffma2(hi2(qv), hi2(x0), ffma2(lo2(qv), lo2(x0), acc[r][0]));
-          }
+          for (int r = 0; r < RW; ++r)
+            acc[r][0] = dot4(*reinterpret_cast<const float4*>(qw + r * D + 4 * c), x0, acc[r][0]);
         }
       }
       // keys past the row's last visible one (their tile rows may hold
       // anything) do not count
 #pragma unroll
       for (int r = 0; r < RW; ++r) {
-        s[r][0] = t0 + lane < vis[r] ? (acc[r][0].x + acc[r][0].y) * a.scale_log2 : -INFINITY;
-        s[r][1] = two && t0 + lane + 32 < vis[r] ? (acc[r][1].x + acc[r][1].y) * a.scale_log2
-                                                 : -INFINITY;
+        s[r][0] = t0 + lane < vis[r] ? acc[r][0] * a.scale_log2 : -INFINITY;
+        s[r][1] = two && t0 + lane + 32 < vis[r] ? acc[r][1] * a.scale_log2 : -INFINITY;
       }
     }
     // ---- softmax of the tile
@@ -366,10 +337,7 @@ attn_f32_kernel(const F32Args a) {
       m[r] = mn;
       l[r] = fmaf(l[r], alpha, p0 + p1);
 #pragma unroll
-      for (int c = 0; c < kPer / 2; ++c) {
-        o[r][c].x *= alpha;
-        o[r][c].y *= alpha;
-      }
+      for (int c = 0; c < kPer; ++c) o[r][c] *= alpha;
       pw[r * kF32Keys + lane] = p0;
       pw[r * kF32Keys + lane + 32] = p1;
     }
@@ -379,26 +347,26 @@ attn_f32_kernel(const F32Args a) {
     // ---- O += P V, 4 keys at a time
 #pragma unroll 2
     for (int j = 0; j < n; j += 4) {
-      float2 v[4][kPer / 2];
+      float v[4][kPer];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         if constexpr (kPer == 4) {
           const float4 x = *reinterpret_cast<const float4*>(v_s + (j + e) * D + 4 * lane);
-          v[e][0] = lo2(x);
-          v[e][kPer / 2 - 1] = hi2(x);
+          v[e][0] = x.x, v[e][1] = x.y, v[e][2] = x.z, v[e][3] = x.w;
         } else {
-          v[e][0] = *reinterpret_cast<const float2*>(v_s + (j + e) * D + 2 * lane);
+          const float2 x = *reinterpret_cast<const float2*>(v_s + (j + e) * D + 2 * lane);
+          v[e][0] = x.x, v[e][1] = x.y;
         }
       }
 #pragma unroll
       for (int r = 0; r < RW; ++r) {
         const float4 p = *reinterpret_cast<const float4*>(pw + r * kF32Keys + j);
 #pragma unroll
-        for (int c = 0; c < kPer / 2; ++c) {
-          o[r][c] = ffma2(make_float2(p.x, p.x), v[0][c], o[r][c]);
-          o[r][c] = ffma2(make_float2(p.y, p.y), v[1][c], o[r][c]);
-          o[r][c] = ffma2(make_float2(p.z, p.z), v[2][c], o[r][c]);
-          o[r][c] = ffma2(make_float2(p.w, p.w), v[3][c], o[r][c]);
+        for (int c = 0; c < kPer; ++c) {
+          o[r][c] = fmaf(p.x, v[0][c], o[r][c]);
+          o[r][c] = fmaf(p.y, v[1][c], o[r][c]);
+          o[r][c] = fmaf(p.z, v[2][c], o[r][c]);
+          o[r][c] = fmaf(p.w, v[3][c], o[r][c]);
         }
       }
     }
@@ -406,13 +374,13 @@ attn_f32_kernel(const F32Args a) {
   }
   grid_dependents_launch();
 
-  auto store_row = [&](int rl, const float2 (&x)[kPer / 2], float inv_of) {
+  auto store_row = [&](int rl, const float (&x)[kPer], float sum) {
     const int r = chunk * kRowsCta + rl;
     if (r >= a.M) return;
     float* dst = a.out + (((size_t)b * a.k + r / a.G) * a.Hq + hkv * a.G + r % a.G) * D + kPer * lane;
 #pragma unroll
-    for (int c = 0; c < kPer / 2; ++c)
-      *reinterpret_cast<float2*>(dst + 2 * c) = make_float2(x[c].x / inv_of, x[c].y / inv_of);
+    for (int c = 0; c < kPer; c += 2)
+      *reinterpret_cast<float2*>(dst + c) = make_float2(x[c] / sum, x[c + 1] / sum);
   };
   if (a.splits == 1) {
 #pragma unroll
@@ -429,8 +397,8 @@ attn_f32_kernel(const F32Args a) {
     const int rl = RW * warp + r;
     const float lr = warp_sum(l[r]);
 #pragma unroll
-    for (int c = 0; c < kPer / 2; ++c)
-      *reinterpret_cast<float2*>(o_s + rl * D + kPer * lane + 2 * c) = o[r][c];
+    for (int c = 0; c < kPer; c += 2)
+      *reinterpret_cast<float2*>(o_s + rl * D + kPer * lane + c) = make_float2(o[r][c], o[r][c + 1]);
     if (lane == 0) {
       st_s[rl] = m[r];
       st_s[kRowsCta + rl] = lr;
@@ -444,17 +412,17 @@ attn_f32_kernel(const F32Args a) {
     const float mx = warp_max(ms);
     const float w = mx == -INFINITY ? (lane < a.splits ? 1.f : 0.f) : exp2f(ms - mx);
     const float lsum = warp_sum(w * ls);
-    float2 acc[kPer / 2];
+    float acc[kPer];
 #pragma unroll
-    for (int c = 0; c < kPer / 2; ++c) acc[c] = make_float2(0.f, 0.f);
+    for (int c = 0; c < kPer; ++c) acc[c] = 0.f;
 #pragma unroll 4
     for (int e = 0; e < a.splits; ++e) {
       const float we = __shfl_sync(0xffffffffu, w, e);
 #pragma unroll
-      for (int c = 0; c < kPer / 2; ++c) {
-        const float2 x = ld_rank2(o_s + rl * D + kPer * lane + 2 * c, e);
-        acc[c].x = fmaf(we, x.x, acc[c].x);
-        acc[c].y = fmaf(we, x.y, acc[c].y);
+      for (int c = 0; c < kPer; c += 2) {
+        const float2 x = ld_rank2(o_s + rl * D + kPer * lane + c, e);
+        acc[c] = fmaf(we, x.x, acc[c]);
+        acc[c + 1] = fmaf(we, x.y, acc[c + 1]);
       }
     }
     store_row(rl, acc, lsum);

@@ -243,36 +243,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
 }
 
 // ------------------------------------------------------------ epilogue math
-__device__ __forceinline__ RowStats shfl_xor_stats(const RowStats& a, int o) {
-  RowStats r;
-  r.m = __shfl_xor_sync(0xffffffffu, a.m, o);
-  r.S = __shfl_xor_sync(0xffffffffu, a.S, o);
-  r.T = __shfl_xor_sync(0xffffffffu, a.T, o);
-  r.best = __shfl_xor_sync(0xffffffffu, a.best, o);
-  r.idx = __shfl_xor_sync(0xffffffffu, a.idx, o);
-  return r;
-}
-
-// Statistics of one logit (this lane's vocabulary id v, one column).
-__device__ __forceinline__ RowStats lane_stats(float z, bool valid, float g, float tau, int v) {
-  RowStats r;
-  r.m = valid ? z * kLog2e : -INFINITY;
-  r.S = valid ? 1.f : 0.f;
-  r.T = 0.f;
-  r.best = valid ? fmaf(tau, g, z) : -INFINITY;
-  r.idx = valid ? v : 0x7fffffff;
-  return r;
-}
-
-// Reduces one column over the 32 lanes of a warp; every lane gets the result.
-__device__ __forceinline__ RowStats warp_column_stats(float z, bool valid, float g, float tau,
-                                                      int v) {
-  RowStats st = lane_stats(z, valid, g, tau, v);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) st = rowstats_merge(st, shfl_xor_stats(st, o));
-  return st;
-}
-
 // Statistics of 16 logit columns over the 32 vocabulary rows of a warp
 // (lane = row, vocabulary id v0 + lane; z the logits, g the Gumbel noise).
 // Two passes: the column maxima of z log2(e) and of the Gumbel score
@@ -1354,105 +1324,318 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
 }
 
 // ------------------------------------------------------------ fp32 SIMT
-// One CTA per 128 vocab rows (thread = row) and the live hidden rows in
-// groups of 32.  W and the group's hidden rows pass through shared memory in
-// chunks of 32 columns, loaded coalesced, so each W element is read from
-// global memory once per group; each thread keeps its 32 logits in
-// registers.  Every logit is still the sequential fp32 FMA chain over H in
-// ascending order (padding columns add 0 * 0).  The same column statistics
-// as the tensor-core epilogue.
+// One CTA per 128 vocabulary rows; the live hidden rows go in groups of up
+// to 32.  W and the group's hidden rows stream through a ring of 4 shared-
+// memory stages of 32 columns (cp.async), so each W element is read from
+// global memory once per group.  A lane holds 8 vocabulary rows of TR hidden
+// rows, a warp 128 x 2 TR logits over a share of every stage's columns: the 8
+// warps split the columns (8 or 16 rows) or the columns and the rows (24 or
+// 32 rows).  TR + 8 shared-memory reads feed 32 TR FMAs.  The partial logits
+// meet in shared memory, and each warp reduces every eighth row over its 128
+// ids (two passes: the maxima, then the sums against them).
+//
+// Bound: W's bytes up to ~16 rows, the FMAs above (128 per SM and cycle).
+// The form before read both operands of every scalar FMA from shared memory
+// with one stage and one thread per vocabulary row.  Per call with the
+// compaction and the merge, V = 32003, H = 2048 (262 MB of W: 39 us; 32 rows
+// of FMAs: 52 us, 63 with the 251 tiles on 152 SMs): 18-30 rows 714-926 us
+// before, 132 now; 16 rows 75, 8 rows 51.  Shared memory returns 128 bytes a
+// cycle to registers, broadcasts included: with 8 rows x 4 ids a lane (12
+// reads for 128 FMAs) the reads bound it (32 rows 148 us).
+constexpr int kF32HeadWarps = 8;
+constexpr int kF32HeadThreads = 32 * kF32HeadWarps;
 constexpr int kF32Cols = 32;
+constexpr int kF32Stages = 4;
+constexpr int kF32Rows = 32;                         // rows of a group
+constexpr int kF32StageFloats = (kBM + kF32Rows) * kF32Cols;
+constexpr size_t kF32SmemBytes = sizeof(float) * kF32Stages * kF32StageFloats;
+static_assert(kF32HeadWarps * 16 * kBM <= kF32Stages * kF32StageFloats, "the partial logits fit the ring");
+
+// The 16-byte column c (of 8) of a staged W row, turned by the row, so that
+// 8 consecutive rows' reads of one column fall into distinct banks.
+__device__ __forceinline__ int f32_w_at(int row, int c) {
+  return row * kF32Cols + (((c ^ row) & 7) << 2);
+}
+
+struct F32HeadTile {
+  const float* w;          // W row v0
+  const float* hidden;     // hidden row r0
+  int H, v_left, rows;     // columns; vocabulary rows from v0; rows to load (past R: zeros)
+};
+
+// Partial logits of the tile into ring as [warp][2 TR rows][kBM], up to 16
+// rows (W's bytes bound it): a ring of 4 stages filled with cp.async, row by
+// row; warp w takes 16-byte column w of every stage.
+template <int TR>
+__device__ __forceinline__ void f32_tile_ring(const F32HeadTile& t, float* ring) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n_chunks = (t.H + kF32Cols - 1) / kF32Cols;
+  const int c_ld = tid & 7, r_ld = tid >> 3;         // staged 16-byte column, first row
+  const int vl = lane & 15;                          // ids vl + 16 j
+  const int row0 = (lane >> 4) * TR;                 // rows row0 + r
+  auto load = [&](int chunk) {
+    float* ws = ring + (chunk % kF32Stages) * kF32StageFloats;
+    float* hs = ws + kBM * kF32Cols;
+    const int col = chunk * kF32Cols + 4 * c_ld;
+    const bool in = col < t.H;
+    const float* wp = t.w + (in ? col : 0);
+#pragma unroll
+    for (int i = 0; i < kBM * 8 / kF32HeadThreads; ++i) {
+      const int row = r_ld + (kF32HeadThreads / 8) * i;
+      const bool ok = in && row < t.v_left;
+      cp_async16(ws + f32_w_at(row, c_ld), ok ? wp + (size_t)row * t.H : t.w, ok);
+    }
+    if (r_ld < t.rows)
+      cp_async16(hs + r_ld * kF32Cols + 4 * c_ld, t.hidden + (size_t)r_ld * t.H + (in ? col : 0), in);
+  };
+#pragma unroll
+  for (int c = 0; c < kF32Stages - 1; ++c) {
+    if (c < n_chunks) load(c);
+    cp_async_commit();
+  }
+  float acc[TR][8];
+#pragma unroll
+  for (int r = 0; r < TR; ++r)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[r][j] = 0.f;
+  for (int chunk = 0; chunk < n_chunks; ++chunk) {
+    cp_async_wait<kF32Stages - 2>();
+    __syncthreads();                                 // chunk landed; chunk - 1 consumed
+    if (chunk + kF32Stages - 1 < n_chunks) load(chunk + kF32Stages - 1);
+    cp_async_commit();
+    const float* ws = ring + (chunk % kF32Stages) * kF32StageFloats;
+    const float* hs = ws + kBM * kF32Cols + row0 * kF32Cols;
+    float4 x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      x[j] = *reinterpret_cast<const float4*>(ws + f32_w_at(vl + 16 * j, warp));
+#pragma unroll
+    for (int r = 0; r < TR; ++r) {
+      const float4 hv = *reinterpret_cast<const float4*>(hs + r * kF32Cols + 4 * warp);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[r][j] = dot4(hv, x[j], acc[r][j]);
+    }
+  }
+  __syncthreads();                                   // every stage consumed
+  float* zs = ring + (warp * 2 * TR + row0) * kBM + vl;
+#pragma unroll
+  for (int r = 0; r < TR; ++r)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) zs[r * kBM + 16 * j] = acc[r][j];
+  __syncthreads();
+}
+
+// The same as [column share][4 TR rows][kBM] above 16 rows (the FMAs bound
+// it): warp w is row group w % 2 and takes 8 columns of every 32, share w / 2.
+// The chunks are transposed on their way through registers into two buffers
+// of shared memory ([column][id] and [column][row], 8-float groups turned by
+// the column against bank conflicts of the stores): an
+// operand register then always meets the same accumulators, which the
+// register allocation can keep in the other bank.  With both operands read
+// along the columns an FMA's operand and accumulator fell into one bank half
+// of the time (dispatch stalls, 48 % of the FMA rate).
+template <int TR>
+__device__ __forceinline__ void f32_tile_cols(const F32HeadTile& t, float* ring) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n_chunks = (t.H + kF32Cols - 1) / kF32Cols;
+  const int c_ld = tid & 7, r_ld = tid >> 3;
+  const int vl = 4 * (lane & 15);                    // ids vl .. + 3 and 64 + vl .. + 3
+  const int row0 = (warp & 1) * 2 * TR + (lane >> 4) * TR;
+  const int part = warp >> 1;
+  constexpr int kIter = kBM * 8 / kF32HeadThreads;
+  constexpr int kBuf = kF32Cols * (kBM + kF32Rows);  // floats of a buffer
+  float4 wr[kIter], hr;
+  auto fetch = [&](int chunk) {
+    const int col = chunk * kF32Cols + 4 * c_ld;
+    const bool in = col < t.H;
+#pragma unroll
+    for (int i = 0; i < kIter; ++i) {
+      const int row = r_ld + (kF32HeadThreads / 8) * i;
+      wr[i] = in && row < t.v_left
+                  ? __ldg(reinterpret_cast<const float4*>(t.w + (size_t)row * t.H + col))
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    hr = in && r_ld < t.rows
+             ? *reinterpret_cast<const float4*>(t.hidden + (size_t)r_ld * t.H + col)
+             : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  const int turn_st = 8 * (c_ld >> 1);               // of columns 4 c_ld .. + 3
+  auto put = [&](float* buf) {
+#pragma unroll
+    for (int i = 0; i < kIter; ++i) {
+      float* d = buf + 4 * c_ld * kBM + ((r_ld + (kF32HeadThreads / 8) * i) ^ turn_st);
+      d[0] = wr[i].x;
+      d[kBM] = wr[i].y;
+      d[2 * kBM] = wr[i].z;
+      d[3 * kBM] = wr[i].w;
+    }
+    float* d = buf + kF32Cols * kBM + 4 * c_ld * kF32Rows + (r_ld ^ turn_st);
+    d[0] = hr.x;
+    d[kF32Rows] = hr.y;
+    d[2 * kF32Rows] = hr.z;
+    d[3 * kF32Rows] = hr.w;
+  };
+  float acc[TR][8];
+#pragma unroll
+  for (int r = 0; r < TR; ++r)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[r][j] = 0.f;
+  // this thread's words of its share's columns 8 part + kk, relative to `at`
+  const int at = 8 * part * kBM;
+  const int x_at = vl ^ (8 * part);
+  int h_at[TR / 2];
+#pragma unroll
+  for (int r = 0; r < TR; r += 2)
+    h_at[r / 2] = kF32Cols * kBM - at + 8 * part * kF32Rows + ((row0 + r) ^ (8 * part));
+  fetch(0);
+  put(ring);
+  if (n_chunks > 1) fetch(1);
+  __syncthreads();
+  for (int chunk = 0; chunk < n_chunks; ++chunk) {
+    const float* buf = ring + (chunk & 1) * kBuf + at;
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+      const float4 x0 = *reinterpret_cast<const float4*>(buf + x_at + kk * kBM);
+      const float4 x1 = *reinterpret_cast<const float4*>(buf + x_at + kk * kBM + 64);
+      const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+      float h[TR];
+#pragma unroll
+      for (int r = 0; r < TR; r += 2) {
+        const float2 v = *reinterpret_cast<const float2*>(buf + h_at[r / 2] + kk * kF32Rows);
+        h[r] = v.x;
+        h[r + 1] = v.y;
+      }
+#pragma unroll
+      for (int r = 0; r < TR; ++r)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[r][j] = fmaf(h[r], xs[j], acc[r][j]);
+    }
+    if (chunk + 1 < n_chunks) {
+      put(ring + ((chunk + 1) & 1) * kBuf);          // consumed before the last barrier
+      if (chunk + 2 < n_chunks) fetch(chunk + 2);
+    }
+    __syncthreads();
+  }
+  float* zs = ring + (part * 4 * TR + row0) * kBM + vl;
+#pragma unroll
+  for (int r = 0; r < TR; ++r) {
+    *reinterpret_cast<float4*>(zs + r * kBM) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+    *reinterpret_cast<float4*>(zs + r * kBM + 64) = make_float4(acc[r][4], acc[r][5], acc[r][6], acc[r][7]);
+  }
+  __syncthreads();
+}
+
 template <bool kPhilox>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kF32HeadThreads, 2)
 head_f32_kernel(const float* __restrict__ hidden_c, const float* __restrict__ w,
                 const float* __restrict__ gumbel, const int32_t* __restrict__ row_map,
                 const int32_t* __restrict__ n_rows, float tau, int V, int H, int rows_alloc,
                 float4* __restrict__ part_msTb, int32_t* __restrict__ part_idx,
                 uint4 philox_sk) {
+  extern __shared__ __align__(16) float f32_smem[];
   grid_dependency_wait();
-  __shared__ float4 sm[4][32];
-  __shared__ int si[4][32];
-  __shared__ float w_s[128][kF32Cols + 1];   // +1: rows land in distinct banks
-  __shared__ float h_s[32][kF32Cols];
   const int R = *n_rows;
-  const int v0 = blockIdx.x * 128;
-  const int v = v0 + threadIdx.x;
-  const bool valid = v < V;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int v0 = blockIdx.x * kBM;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool noisy = tau != 0.f && (kPhilox || gumbel != nullptr);
-  for (int r0 = 0; r0 < R; r0 += 32) {
-    const int nr = min(32, R - r0);
-    float zr[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) zr[j] = 0.f;
-    for (int c0 = 0; c0 < H; c0 += kF32Cols) {
-      const int nc = min(kF32Cols, H - c0);
-      __syncthreads();   // the previous chunk is consumed
-      for (int e = threadIdx.x; e < 128 * kF32Cols; e += 128) {
-        const int rr = e / kF32Cols, cc = e % kF32Cols;
-        w_s[rr][cc] = (v0 + rr < V && cc < nc) ? w[(size_t)(v0 + rr) * H + c0 + cc] : 0.f;
-      }
-      for (int e = threadIdx.x; e < 32 * kF32Cols; e += 128) {
-        const int jj = e / kF32Cols, cc = e % kF32Cols;
-        h_s[jj][cc] = (jj < nr && cc < nc) ? hidden_c[(size_t)(r0 + jj) * H + c0 + cc] : 0.f;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        if (j < nr) {
-          float acc = zr[j];
-#pragma unroll 8
-          for (int cc = 0; cc < kF32Cols; ++cc) acc = fmaf(h_s[j][cc], w_s[threadIdx.x][cc], acc);
-          zr[j] = acc;
-        }
-      }
+  const int vq = v0 + 4 * lane;                      // this lane's first id in the reduction
+
+  for (int r0 = 0; r0 < R; r0 += kF32Rows) {
+    const int nr = min(kF32Rows, R - r0);
+    F32HeadTile t;
+    t.w = w + (size_t)v0 * H;
+    t.hidden = hidden_c + (size_t)r0 * H;
+    t.H = H;
+    t.v_left = V - v0;
+    t.rows = (nr + 7) & ~7;                          // hidden_c has zero rows past R
+    int zrows = 32, parts = 4;                       // [parts][zrows][kBM] partial logits
+    if (nr <= 8) {
+      f32_tile_ring<4>(t, f32_smem);
+      zrows = 8, parts = 8;
+    } else if (nr <= 16) {
+      f32_tile_ring<8>(t, f32_smem);
+      zrows = 16, parts = 8;
+    } else if (nr <= 24) {
+      f32_tile_cols<6>(t, f32_smem);
+      zrows = 24;
+    } else {
+      f32_tile_cols<8>(t, f32_smem);
     }
-    RowStats mine = rowstats_empty();
+    const float* zs = f32_smem;
+    // noise of this warp's rows warp, warp + 8, ... of the group
+    float g[kF32Rows / kF32HeadWarps][4];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      if (j >= nr) break;
-      const float z = zr[j];
-      float g = 0.f;
-      if (noisy && valid) {
+    for (int i = 0; i < kF32Rows / kF32HeadWarps; ++i) {
+      const int row = warp + kF32HeadWarps * i;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) g[i][j] = 0.f;
+      if (noisy && row < nr) {
+        const int n = row_map[r0 + row];
         if constexpr (kPhilox) {
-          // philox_sk = (seed low, seed high, offset low, offset high)
+          // philox_sk = (seed low, seed high, offset low, offset high); the
+          // lane's four ids are the four words of one call
           const uint4 x = sbd_philox::philox4x32_10(
-              make_uint4((uint32_t)v >> 2, (uint32_t)row_map[r0 + j], philox_sk.z, philox_sk.w),
-              philox_sk.x, philox_sk.y);
-          g = sbd_philox::gumbel_of_word(sbd_philox::word_of(x, v & 3));
+              make_uint4((uint32_t)vq >> 2, (uint32_t)n, philox_sk.z, philox_sk.w), philox_sk.x,
+              philox_sk.y);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) g[i][j] = sbd_philox::gumbel_of_word(sbd_philox::word_of(x, j));
         } else {
-          g = gumbel[(size_t)row_map[r0 + j] * V + v];
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (vq + j < V) g[i][j] = __ldg(gumbel + (size_t)n * V + vq + j);
         }
       }
-      const RowStats cs = warp_column_stats(z, valid, g, tau, v);
-      if (lane == j) mine = cs;
     }
-    if (lane < nr) {
-      sm[warp][lane] = make_float4(mine.m, mine.S, mine.T, mine.best);
-      si[warp][lane] = mine.idx;
-    }
-    __syncthreads();
-    if (threadIdx.x < nr) {
-      RowStats s;
-      s.m = sm[0][threadIdx.x].x;
-      s.S = sm[0][threadIdx.x].y;
-      s.T = sm[0][threadIdx.x].z;
-      s.best = sm[0][threadIdx.x].w;
-      s.idx = si[0][threadIdx.x];
-      for (int w2 = 1; w2 < 4; ++w2) {
-        RowStats o;
-        o.m = sm[w2][threadIdx.x].x;
-        o.S = sm[w2][threadIdx.x].y;
-        o.T = sm[w2][threadIdx.x].z;
-        o.best = sm[w2][threadIdx.x].w;
-        o.idx = si[w2][threadIdx.x];
-        s = rowstats_merge(s, o);
+#pragma unroll
+    for (int i = 0; i < kF32Rows / kF32HeadWarps; ++i) {
+      const int row = warp + kF32HeadWarps * i;
+      if (row >= nr) break;
+      float z[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int p = 0; p < parts; ++p) {
+        const float4 x = *reinterpret_cast<const float4*>(zs + (p * zrows + row) * kBM + 4 * lane);
+        z[0] += x.x;
+        z[1] += x.y;
+        z[2] += x.z;
+        z[3] += x.w;
       }
-      const size_t o = (size_t)blockIdx.x * rows_alloc + r0 + threadIdx.x;
-      part_msTb[o] = make_float4(s.m, s.S, s.T, s.best);
-      part_idx[o] = s.idx;
+      float y[4], mx = -INFINITY, best = -INFINITY;
+      int idx = vq;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bool ok = vq + j < V;
+        y[j] = z[j] * kLog2e;
+        if (ok) mx = fmaxf(mx, y[j]);
+        const float sc = fmaf(tau, g[i][j], z[j]);
+        if (ok && sc > best) {                       // ids ascend: the lowest wins ties
+          best = sc;
+          idx = vq + j;
+        }
+      }
+      const float m = warp_max(mx);
+      const float wbest = warp_max(best);
+      // the lowest lane that reaches the best score (lane 0's first id when
+      // no score compares, i.e. every logit is NaN)
+      const unsigned hits = __ballot_sync(0xffffffffu, vq < V && best == wbest);
+      const int win = __shfl_sync(0xffffffffu, idx, hits ? __ffs(hits) - 1 : 0);
+      float S = 0.f, T = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (vq + j < V) {
+          const float d = y[j] - m;                  // <= 0
+          const float e = exp2f(d);
+          S += e;
+          T = fmaf(e, d, T);
+        }
+      }
+      S = warp_sum(S);
+      T = warp_sum(T);
+      if (lane == 0) {
+        const size_t o = (size_t)blockIdx.x * rows_alloc + r0 + row;
+        part_msTb[o] = make_float4(m, S, T, wbest);
+        part_idx[o] = win;
+      }
     }
-    __syncthreads();
+    __syncthreads();                                 // the partial logits are read
   }
 }
 
@@ -1791,7 +1974,9 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
                     (void*)&pi, (void*)&sk};
     const void* fn =
         philox ? (const void*)head_f32_kernel<true> : (const void*)head_f32_kernel<false>;
-    s = launch_pdl(fn, dim3(p.n_ctas), dim3(128), 0, st, args, "head_f32_kernel launch");
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32SmemBytes);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(head_f32_kernel)");
+    s = launch_pdl(fn, dim3(p.n_ctas), dim3(kF32HeadThreads), kF32SmemBytes, st, args, "head_f32_kernel launch");
     if (s != SBD_OK) return s;
   }
   {

@@ -286,6 +286,26 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// ---- fp32 kernels
+// acc + a . b, in ascending order.  (Scalar FMAs: the packed fma.rn.f32x2
+// reads three register pairs an instruction and reached 48 TFLOP/s in an
+// 8 x 4 outer product, scalar FMAs 68 in 8 x 8, on GB300.)
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float acc) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
+}
+// 16 bytes global -> shared, asynchronously; zeros when !valid (src is not read).
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 // Running statistics of one logit row over a subset of the vocabulary, in
 // base-2 units (y = z * log2 e):  m = max y,  S = sum 2^(y-m),
 // T = sum 2^(y-m) (y-m); plus the best Gumbel score and its vocabulary id.

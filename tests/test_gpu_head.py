@@ -79,6 +79,32 @@ def test_f32_random_shapes(sbd, case):
     assert compare_head(d, "f32", tau, ent, tok, with_noise=tau != 0.0) <= 1
 
 
+@pytest.mark.parametrize("philox", [False, True])
+@pytest.mark.parametrize("V,H", [(1, 4), (127, 28), (129, 32), (261, 100)])
+@pytest.mark.parametrize("R", [1, 8, 9, 16, 17, 24, 25, 32, 33, 41, 64])
+def test_f32_row_groups(sbd, R, V, H, philox):
+    """Exactly R masked rows of 64 through head_f32_kernel: the edges of its
+    row counts per group (8, 16, 24, 32), one id, one id past a tile, column
+    counts around the 32-column stage; noise from the buffer and the kernel's
+    own, which must agree bit for bit."""
+    import torch
+    w = gen.shrink(gen.get_workload("tiny_f32"), batch=4, block_k=16, vocab=V, hidden=H)
+    d = dict(step_inputs(w, seed=R))
+    m = np.zeros(64, dtype=np.uint8)
+    m[np.random.default_rng(R).choice(64, size=R, replace=False)] = 1
+    d["masked"] = m.reshape(4, 16)
+    if philox:
+        ids = torch.arange(64, dtype=torch.int32, device="cuda")
+        d["gumbel"] = sbd.sbd_gumbel_philox(ids, V, 9, 3).cpu().numpy().reshape(4, 16, V)
+    ent, tok = run_head(sbd, d, "f32", 1.0)
+    assert compare_head(d, "f32", 1.0, ent, tok) <= 1
+    if philox:
+        e2, t2 = sbd.sbd_head_entropy_sample_philox(
+            to_dev(d["hidden"], "f32"), to_dev(d["w"], "f32"), torch.from_numpy(d["masked"]).cuda(), 9, 3, 1.0)
+        assert np.array_equal(t2.cpu().numpy(), tok) and np.array_equal(e2.cpu().numpy(), ent)
+    assert sbd.sbd_device_error() == 0
+
+
 @pytest.mark.parametrize("B,k,V,H", [(1, 1, 1000, 256), (1, 16, 4096 + 5, 512), (2, 16, 3000, 128),
                                      (3, 7, 777, 64), (16, 16, 2100, 256), (1, 17, 500, 128),
                                      (10, 30, 999, 64), (16, 32, 1500, 128),
