@@ -65,6 +65,10 @@ constexpr int kEpiWarps = 8;
 // spills registers.
 constexpr int kGAhead = 3;
 constexpr int kEpiThreads = 32 * kEpiWarps;
+// kLinear: K ranges of a cluster at most, and stages per range at least for
+// the longer stages (so that whole stages split evenly).
+constexpr int kMaxRanges = 8;
+constexpr int kRangeStages = 4;
 constexpr int kHeadThreads = 64 + kEpiThreads;   // warp 0 TMA, warp 1 MMA, then the epilogue
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -242,6 +246,31 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
   }
 }
 
+// 16 bytes at the shared-memory address `addr` of CTA `rank` of the cluster.
+__device__ __forceinline__ float4 ld_cta_v4(uint32_t addr, int rank) {
+  uint32_t p;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(p)
+               : "memory");
+  return v;
+}
+
+// Two values rounded to bf16 (nearest even), the first in the low half.
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// 32 bytes to global memory (a whole sector) in one store.
+__device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]),
+               "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
 // ------------------------------------------------------------ epilogue math
 // Statistics of 16 logit columns over the 32 vocabulary rows of a warp
 // (lane = row, vocabulary id v0 + lane; z the logits, g the Gumbel noise).
@@ -399,6 +428,7 @@ struct HeadArgs {
   __nv_bfloat16* y;     // kLinear: output [linear_rows, V]
   int linear_rows;      // kLinear: rows of x, all live
   int ksplit;           // kLinear: K ranges per output tile (1: y written directly)
+  int k_cluster;        // kLinear: the ranges of a tile form one cluster and add up there
   float* part_y;        // kLinear, ksplit > 1: fp32 partials [ksplit][linear_rows][V]
 };
 
@@ -428,6 +458,18 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
     tma_prefetch_desc(&tmap_h);
   }
   if (warp == 1) tc_alloc(&tmem_base_sh, a.tmem_cols);
+  if constexpr (kLinear) {
+    // Nothing says that the previous kernel on the stream did not write W, so
+    // it is not read before that kernel is done; but its first boxes come into
+    // L2 (which stays coherent) meanwhile.  With the early trigger below, the
+    // four GEMMs of an 8B layer in turn took 90.5 -> 87.4 us at 16 rows,
+    // 138.2 -> 128.6 at 160, 171.3 -> 167.0 at 512 (24 boxes: 89.3, 6: 88.1).
+    if (warp == 0 && lane < 12) {
+      const int kb = (a.H / kBK) * (int)(blockIdx.x % a.ksplit) / a.ksplit + lane;
+      if (kb < a.H / kBK)
+        tma_prefetch_l2_2d(&tmap_w, kb * kBK, (int)(blockIdx.x / a.ksplit) * kBM);
+    }
+  }
   // Everything below reads what the compaction kernel wrote.
   grid_dependency_wait();
   const int R = kLinear ? a.linear_rows : *a.n_rows;
@@ -467,7 +509,8 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
   auto fits = [&](int bx, int n_st) { return ring_bytes / (bx * (kABytes + b_box)) >= n_st; };
   int boxes = kMaxBoxes;
   while (boxes > 1 &&
-         ((a.H / kBK) % (boxes * ksplit) != 0 || !fits(boxes, boxes > 2 ? 3 : 2)))
+         ((a.H / kBK) % boxes != 0 || !fits(boxes, boxes > 2 ? 3 : 2) ||
+          (ksplit > 1 && (a.H / kBK) / boxes < kRangeStages * ksplit)))
     boxes >>= 1;
   const int stage_bytes = boxes * (kABytes + b_box);     // [A boxes | B boxes]
   int stages = ring_bytes / stage_bytes;
@@ -498,7 +541,9 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
-  const int num_kb = a.H / (kBK * boxes) / ksplit;   // stages per unit
+  // the stages of K range ks: kb_of(ks) .. kb_of(ks + 1) - 1
+  const int num_st = a.H / (kBK * boxes);
+  auto kb_of = [&](int ks) { return ksplit == 1 ? ks * num_st : ks * num_st / ksplit; };
 
   if (R > 0) {
     if (warp == 0) {
@@ -511,8 +556,8 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
         uint32_t ph = 0;
         bool ok = true;
         for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-          const int tile = u / ksplit, kb0 = (u % ksplit) * num_kb;
-          for (int kb = 0; kb < num_kb; ++kb, ++it) {
+          const int tile = u / ksplit, ks = u % ksplit;
+          for (int kb = kb_of(ks); kb < kb_of(ks + 1); ++kb, ++it) {
             if (!mbar_wait(&empty_bar[s], ph ^ 1, a.err)) {
               ok = false;
               break;
@@ -520,7 +565,7 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
             uint8_t* st = ring + (size_t)s * stage_bytes;
             mbar_arrive_expect_tx(&full_bar[s], stage_bytes);
             for (int x = 0; x < boxes; ++x) {
-              const int col = ((kb0 + kb) * boxes + x) * kBK;
+              const int col = (kb * boxes + x) * kBK;
               tma_load_2d_hint(st + x * kABytes, &tmap_w, &full_bar[s], col, tile * kBM, policy);
               // the n_eff hidden rows the MMA reads, in the tallest boxes that
               // fit: these rows come from L2 for every vocabulary tile, where
@@ -541,6 +586,8 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
             }
           }
         }
+        // every copy is issued: the next kernel may come up and prefetch
+        if constexpr (kLinear) grid_dependents_launch();
         // copies still in flight must land before the CTA exits
         for (int q = it - stages > 0 ? it - stages : 0; q < it; ++q)
           mbar_wait(&full_bar[q % stages], (q / stages) & 1, a.err);
@@ -561,7 +608,8 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
           if (!mbar_wait(&tmem_empty[acc], (use & 1) ^ 1, a.err)) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + (uint32_t)acc * acc_stride;
-          for (int kb = 0; kb < num_kb; ++kb, ++it) {
+          const int kb0 = kb_of(u % ksplit), kb1 = kb_of(u % ksplit + 1);
+          for (int kb = kb0; kb < kb1; ++kb, ++it) {
             if (!mbar_wait(&full_bar[s], ph, a.err)) {
               ok = false;
               break;
@@ -573,7 +621,7 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
               const uint64_t bdesc = sw128_kmajor_desc(st + boxes * kABytes + x * b_box);
 #pragma unroll
               for (int kk = 0; kk < kBK / 16; ++kk) {
-                const uint32_t accum = (kb != 0 || x != 0 || kk != 0);
+                const uint32_t accum = (kb != kb0 || x != 0 || kk != 0);
                 tc_mma_bf16(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc_lo, accum);
                 if (n_hi > 0)   // rows 256.. of B: 256 x 128 B further on, 256 columns on
                   tc_mma_bf16(d_tmem + 256, adesc + 2 * kk, bdesc + (256 * 128 >> 4) + 2 * kk,
@@ -672,7 +720,14 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
           if constexpr (kLinear) {
             // y[c0 + j, v] (or its fp32 partial of K range ks): for each j the
             // warp's lanes store 32 consecutive v
-            if (valid) {
+            if (a.k_cluster) {
+              // the range's partial, [row][vocabulary row of the tile], over
+              // the ring: every stage was consumed before tmem_full
+              float* pz = reinterpret_cast<float*>(ring) + c0 * kBM + quad * 32 + lane;
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                if (c0 + j < R) pz[j * kBM] = __uint_as_float(r[j]);
+            } else if (valid) {
               if (ksplit == 1) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
@@ -717,6 +772,45 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
   if (warp == 1) {
     tc_fence_after();
     tc_dealloc(tmem_base, a.tmem_cols);
+  }
+  if constexpr (kLinear) {
+    if (a.k_cluster) {
+      // y = the sum over the cluster's ranges, in range order: CTA `ks` takes
+      // rows ks, ks + ksplit, ..., a warp a row, a lane 4 outputs.  The second
+      // barrier keeps every CTA's partial alive until the others have read it.
+      pair_sync();
+      const int ks = (int)(blockIdx.x % ksplit), v0 = (int)(blockIdx.x / ksplit) * kBM + 4 * lane;
+      const uint32_t zb = smem_u32(ring) + 16u * lane;
+      const bool vec = a.V % 4 == 0 && v0 + 4 <= a.V;
+      for (int r = ks + ksplit * warp; r < R; r += ksplit * (kHeadThreads / 32)) {
+        float4 v[kMaxRanges];
+#pragma unroll
+        for (int e = 0; e < kMaxRanges; ++e)
+          if (e < ksplit) v[e] = ld_cta_v4(zb + (uint32_t)(r * kBM * 4), e);
+        float4 acc = v[0];
+#pragma unroll
+        for (int e = 1; e < kMaxRanges; ++e)
+          if (e < ksplit) {
+            acc.x += v[e].x;
+            acc.y += v[e].y;
+            acc.z += v[e].z;
+            acc.w += v[e].w;
+          }
+        __nv_bfloat16* y = a.y + (size_t)r * a.V + v0;
+        if (vec) {
+          uint2 w;
+          w.x = pack_bf16x2(acc.x, acc.y);
+          w.y = pack_bf16x2(acc.z, acc.w);
+          *reinterpret_cast<uint2*>(y) = w;
+        } else {
+          const float o[4] = {acc.x, acc.y, acc.z, acc.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (v0 + j < a.V) y[j] = __float2bfloat16_rn(o[j]);
+        }
+      }
+      pair_sync();
+    }
   }
 }
 
@@ -802,12 +896,6 @@ __device__ __forceinline__ void fold_chunk16(RowStats& st, const float (&z)[16],
 // always in the rows layout, the epilogue storing each row's outputs; with
 // a.ksplit > 1 each (pair tile, K range) is a unit and the epilogue stores
 // fp32 partials for linear_reduce_kernel.
-// Two values rounded to bf16 (nearest even), the first in the low half.
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
-
 template <bool kPhilox, bool kLinear>
 __global__ void __launch_bounds__(kHeadThreads, 1)
 head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
@@ -834,6 +922,15 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmap_w);
     tma_prefetch_desc(&tmap_h);
+  }
+  if constexpr (kLinear) {
+    // W's first boxes into L2 while the previous kernel finishes (see head_tc_kernel)
+    if (warp == 0 && lane < 6) {
+      const int tk = pair / (a.linear_rows > 2 * kPairRows ? 2 : 1);
+      const int kb = (a.H / kBK) / a.ksplit * (tk % a.ksplit) + lane;
+      if (kb < a.H / kBK)
+        tma_prefetch_l2_2d(&tmap_w, kb * kBK, (2 * (tk / a.ksplit) + rank) * kBM);
+    }
   }
   // Everything below reads what the compaction kernel wrote.
   grid_dependency_wait();
@@ -932,7 +1029,11 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
   pair_sync();
   if (warp == 1) tc_alloc_pair(&tmem_base_sh, 512);
   tc_fence_before();
-  __syncthreads();
+  // The producer warp only arrives: its copies need no tensor memory.  (In
+  // the vocabulary layout with in-kernel noise 2-3 % faster than a full
+  // barrier: 131 rows 203.1 -> 195.9 us; elsewhere within 0.5 %.)
+  if (warp == 0) asm volatile("bar.arrive 2, %0;" ::"n"(kHeadThreads) : "memory");
+  else asm volatile("bar.sync 2, %0;" ::"n"(kHeadThreads) : "memory");
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
 
@@ -986,6 +1087,8 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
             }
           }
         }
+        // every copy is issued: the next kernel may come up and prefetch
+        if constexpr (kLinear) grid_dependents_launch();
         // Copies still in flight must land before the CTA exits.  Rank 1
         // cannot wait on rank 0's full barriers: it waits until the MMAs
         // released its last stages, which they do only after they arrived.
@@ -1050,9 +1153,10 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
       const int n = !kLinear && row_live ? a.row_map[h] : 0;
       const bool noisy = !kLinear && a.tau != 0.f && (kPhilox || a.gumbel != nullptr);
       const float* grow = noisy && !kPhilox ? a.gumbel + (size_t)n * a.V : nullptr;
-      // kLinear: 16-byte stores of 8 outputs where the row stride allows
-      const bool y_vec = ((reinterpret_cast<uintptr_t>(a.y) | (uintptr_t)a.V * 2u) & 15u) == 0;
-      const bool p_vec = ((reinterpret_cast<uintptr_t>(a.part_y) | (uintptr_t)a.V * 4u) & 15u) == 0;
+      // kLinear: 32-byte stores where base and row stride allow (each lane
+      // writes its own row: 16-byte stores half-fill every sector)
+      const bool y_vec = ((reinterpret_cast<uintptr_t>(a.y) | (uintptr_t)a.V * 2u) & 31u) == 0;
+      const bool p_vec = ((reinterpret_cast<uintptr_t>(a.part_y) | (uintptr_t)a.V * 4u) & 31u) == 0;
       const bool vec4 = ((reinterpret_cast<uintptr_t>(a.gumbel) | (uintptr_t)a.V * 4u) & 15u) == 0;
       const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
       constexpr int kChunks = 2 * kBM / 16 / 2;   // chunks of one warp per unit
@@ -1133,9 +1237,11 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
                   float* pr = a.part_y + ((size_t)ks * R + h) * a.V + n0;
                   if (p_vec && n0 + 16 <= a.V) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                      reinterpret_cast<float4*>(pr)[i] =
-                          make_float4(z[4 * i], z[4 * i + 1], z[4 * i + 2], z[4 * i + 3]);
+                    for (int i = 0; i < 2; ++i) {
+                      const uint32_t q[8] = {r[8 * i],     r[8 * i + 1], r[8 * i + 2], r[8 * i + 3],
+                                             r[8 * i + 4], r[8 * i + 5], r[8 * i + 6], r[8 * i + 7]};
+                      st_global_v8(pr + 8 * i, q);
+                    }
                   } else {
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
@@ -1144,17 +1250,11 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
                 } else {
                   __nv_bfloat16* yr = a.y + (size_t)h * a.V + n0;
                   if (y_vec && n0 + 16 <= a.V) {
-                    uint4 q0, q1;
-                    q0.x = pack_bf16x2(z[0], z[1]);
-                    q0.y = pack_bf16x2(z[2], z[3]);
-                    q0.z = pack_bf16x2(z[4], z[5]);
-                    q0.w = pack_bf16x2(z[6], z[7]);
-                    q1.x = pack_bf16x2(z[8], z[9]);
-                    q1.y = pack_bf16x2(z[10], z[11]);
-                    q1.z = pack_bf16x2(z[12], z[13]);
-                    q1.w = pack_bf16x2(z[14], z[15]);
-                    reinterpret_cast<uint4*>(yr)[0] = q0;
-                    reinterpret_cast<uint4*>(yr)[1] = q1;
+                    const uint32_t q[8] = {pack_bf16x2(z[0], z[1]),   pack_bf16x2(z[2], z[3]),
+                                           pack_bf16x2(z[4], z[5]),   pack_bf16x2(z[6], z[7]),
+                                           pack_bf16x2(z[8], z[9]),   pack_bf16x2(z[10], z[11]),
+                                           pack_bf16x2(z[12], z[13]), pack_bf16x2(z[14], z[15])};
+                    st_global_v8(yr, q);
                   } else {
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
@@ -1783,17 +1883,39 @@ int head_pair_slots(const void* fn) {
   return clusters;
 }
 
-// y = the sum over K ranges of the fp32 partials of sbd_linear, in bf16.
+// y = the sum over K ranges of the fp32 partials of sbd_linear, in bf16, each
+// element in range order.  kVec: 4 outputs a thread (16-byte reads, every
+// range of the group of 4 in flight), for T N a multiple of 4, where every
+// range starts on 16 bytes; otherwise one output a thread.  (One output a
+// thread took 10 us for 2 ranges of 512 x 4096, ~4 with 4; their
+// 21 MB, out of L2, are 3.1 us of HBM time.)
+template <bool kVec>
 __global__ void __launch_bounds__(256)
 linear_reduce_kernel(const float* __restrict__ part, int ksplit, long long tn,
                      __nv_bfloat16* __restrict__ y) {
   grid_dependency_wait();
   grid_dependents_launch();
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * (kVec ? 4 : 1);
   if (i >= tn) return;
-  float acc = 0.f;
-  for (int ks = 0; ks < ksplit; ++ks) acc += part[(size_t)ks * tn + i];
-  y[i] = __float2bfloat16_rn(acc);
+  if constexpr (kVec) {
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int ks = 0; ks < ksplit; ++ks) {
+      const float4 v = *reinterpret_cast<const float4*>(part + (size_t)ks * tn + i);
+      acc.x += v.x;
+      acc.y += v.y;
+      acc.z += v.z;
+      acc.w += v.w;
+    }
+    uint2 w;
+    w.x = pack_bf16x2(acc.x, acc.y);
+    w.y = pack_bf16x2(acc.z, acc.w);
+    *reinterpret_cast<uint2*>(y + i) = w;
+  } else {
+    float acc = 0.f;
+    for (int ks = 0; ks < ksplit; ++ks) acc += part[(size_t)ks * tn + i];
+    y[i] = __float2bfloat16_rn(acc);
+  }
 }
 
 }  // namespace
@@ -1913,6 +2035,7 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     a.y = nullptr;
     a.linear_rows = 0;
     a.ksplit = 1;
+    a.k_cluster = 0;
     a.part_y = nullptr;
     a.h_big = p.rows_alloc >= 128 ? 128 : (p.rows_alloc >= 64 ? 64 : 16);
     a.tau = tau;
@@ -2065,6 +2188,20 @@ static int pair_linear_ksplit(int T, int K, int N, int n_pairs) {
   return best;
 }
 
+// K ranges of the single-CTA linear kernel's tiles as clusters, all running at
+// once (1: no split): as many as the SMs hold, each at least 4 column blocks.
+// The ranges then add up through distributed shared memory, with no fp32
+// partials in HBM and no second kernel: 4096 -> 6144 columns at 128 rows
+// 21.2 -> 18.0 us, at 160 rows 25.8 -> 20.8; at 16 rows within 0.3 us.
+static int linear_cluster_ranges(const void* fn, size_t smem, int T, int K, int n_tiles) {
+  if (T > kPairVocabLanesMax) return 1;   // T x 128 partials fit the ring
+  for (int ks = kMaxRanges; ks > 1; --ks)
+    if (n_tiles * ks <= num_sms() && K / kBK >= 4 * ks &&
+        cluster_slots(fn, kHeadThreads, smem, ks) >= n_tiles)
+      return ks;
+  return 1;
+}
+
 size_t linear_workspace_bytes(int T, int K, int N) {
   const int ks = linear_max_split(T, K, N);
   return ks > 1 ? (size_t)ks * T * N * sizeof(float) : 0;
@@ -2113,6 +2250,7 @@ sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void
   a.H = K;
   a.rows_alloc = rows_alloc;
   a.n_tiles = (N + kBM - 1) / kBM;
+  a.k_cluster = 0;
   a.h_big = T >= 128 ? 128 : (T >= 64 ? 64 : 16);
   a.tau = 0.f;
   a.y = (__nv_bfloat16*)y;
@@ -2156,24 +2294,33 @@ sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void
     while (cols < (uint32_t)(n_acc_alloc * rows_alloc)) cols <<= 1;
     a.tmem_cols = cols;
     const int slots = num_sms();
+    const int in_cluster = linear_cluster_ranges(fn, smem, T, K, a.n_tiles);
+    if (in_cluster > 1) {
+      ksplit = in_cluster;
+      a.k_cluster = 1;
+      cluster = ksplit;
+    }
     const int units = a.n_tiles * ksplit;
-    n_ctas = units < slots ? units : slots;
+    n_ctas = a.k_cluster || units < slots ? units : slots;
   }
   a.ksplit = ksplit;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(linear kernel)");
   void* args[] = {(void*)&tw, (void*)&tx, (void*)&tx64, (void*)&tx128, (void*)&a};
   s = launch_pdl(fn, dim3(n_ctas), dim3(kHeadThreads), smem, st, args,
-                 cluster > 1 ? "head_pair_kernel (linear) launch" : "head_tc_kernel (linear) launch",
+                 T > kPairVocabLanesMax ? "head_pair_kernel (linear) launch" : "head_tc_kernel (linear) launch",
                  cluster);
-  if (s != SBD_OK || ksplit == 1) return s;
+  if (s != SBD_OK || ksplit == 1 || a.k_cluster) return s;
   const float* part = (const float*)ws;
   long long tn = (long long)T * N;
   __nv_bfloat16* yb = (__nv_bfloat16*)y;
   int ks = ksplit;
   void* rargs[] = {(void*)&part, (void*)&ks, (void*)&tn, (void*)&yb};
-  return launch_pdl((const void*)linear_reduce_kernel, dim3((unsigned)((tn + 255) / 256)), dim3(256),
-                    0, st, rargs, "linear_reduce_kernel launch");
+  const bool vec = tn % 4 == 0;
+  const long long threads = vec ? tn / 4 : tn;
+  return launch_pdl(vec ? (const void*)linear_reduce_kernel<true> : (const void*)linear_reduce_kernel<false>,
+                    dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, rargs,
+                    "linear_reduce_kernel launch");
 }
 
 }  // namespace sbd

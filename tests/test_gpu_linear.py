@@ -47,6 +47,30 @@ def test_matches_fp64_product(sbd, T, K, N):
     assert sbd.sbd_device_error() == 0
 
 
+@pytest.mark.parametrize("T,K,N", [
+    # up to 160 rows: K ranges of a tile in one cluster, 2 to 8 of them, of unequal length, outputs that
+    # end inside a group of four; one range where the tiles fill the SMs
+    (1, 64 * 37, 700), (16, 64 * 33, 1030), (33, 64 * 8, 5), (160, 64 * 9, 130), (160, 64 * 67, 4099),
+    (128, 64 * 21, 6145), (7, 64 * 16, 9730), (16, 64 * 5, 20000),
+    # CTA pairs: unit widths from 2 x 128 down, with and without K ranges; a second row group of one row
+    (161, 64 * 40, 6144), (200, 64 * 12, 4096), (256, 64 * 64, 2050), (257, 64 * 16, 9001),
+    (385, 64 * 8, 4096), (512, 64 * 32, 6144), (512, 64 * 3, 28672)])
+def test_split_and_unit_edges(sbd, T, K, N):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(T + N)
+    x = torch.randn(T, K, generator=g, device="cuda").to(torch.bfloat16)
+    w = (torch.randn(N, K, generator=g, device="cuda") * 0.02).to(torch.bfloat16)
+    y = torch.full((T + 1, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    sbd.sbd_linear(x, w, out=y[:T])
+    ref = x.double() @ w.double().T
+    # half a unit in the last place of the output, plus K fp32 additions of the products
+    bound = x.double().abs() @ w.double().abs().T
+    tol = 2.0 ** -8 * ref.abs() + K * 2.0 ** -23 * bound + 1e-6
+    assert bool(((y[:T].double() - ref).abs() <= tol).all())
+    assert bool((y[T] == 7.0).all())
+    assert sbd.sbd_device_error() == 0
+
+
 def test_out_of_range_rows_are_not_written(sbd):
     import torch
     rng = np.random.default_rng(1)
