@@ -428,6 +428,7 @@ struct HeadArgs {
   __nv_bfloat16* y;     // kLinear: output [linear_rows, V]
   int linear_rows;      // kLinear: rows of x, all live
   int ksplit;           // kLinear: K ranges per output tile (1: y written directly)
+  int w_rows;           // kLinear, pairs: W rows of a unit per CTA (a multiple of 16 up to 128)
   int k_cluster;        // kLinear: the ranges of a tile form one cluster and add up there
   float* part_y;        // kLinear, ksplit > 1: fp32 partials [ksplit][linear_rows][V]
 };
@@ -923,13 +924,17 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
     tma_prefetch_desc(&tmap_w);
     tma_prefetch_desc(&tmap_h);
   }
+  // W rows of a unit in each CTA (head: 128)
+  const int w_rows = kLinear ? a.w_rows : kBM;
   if constexpr (kLinear) {
-    // W's first boxes into L2 while the previous kernel finishes (see head_tc_kernel)
+    // W does not depend on the previous kernel in practice, but nothing says
+    // so: its first boxes are brought into L2 only, which stays coherent, while
+    // that kernel finishes (see head_tc_kernel)
     if (warp == 0 && lane < 6) {
       const int tk = pair / (a.linear_rows > 2 * kPairRows ? 2 : 1);
       const int kb = (a.H / kBK) / a.ksplit * (tk % a.ksplit) + lane;
       if (kb < a.H / kBK)
-        tma_prefetch_l2_2d(&tmap_w, kb * kBK, (2 * (tk / a.ksplit) + rank) * kBM);
+        tma_prefetch_l2_2d(&tmap_w, kb * kBK, (2 * (tk / a.ksplit) + rank) * w_rows);
     }
   }
   // Everything below reads what the compaction kernel wrote.
@@ -975,28 +980,32 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
   uint8_t* ring = gbase + ep_bytes;
   const uint32_t rbase = sbase + (uint32_t)ep_bytes;
   const int ring_bytes = a.ring_bytes - ep_bytes;
-  const int h_box = rows_mode ? ((live_rows(grp * 2 * kPairRows) + 15) / 16 * 16) * kBK * 2
-                              : (G / 2) * kBK * 2;
+  // (with fewer W rows a unit, a hidden box always takes 128 rows: the W boxes
+  // behind the last one may not cover the 128 rows that the MMA reads)
+  const int w_bytes = w_rows * kBK * 2;
+  const int h_box = kLinear && w_rows < kBM ? kPairRows * kBK * 2
+                    : rows_mode ? ((live_rows(grp * 2 * kPairRows) + 15) / 16 * 16) * kBK * 2
+                                : (G / 2) * kBK * 2;
   // At least three stages.  (Two stages of longer W runs had measured 1-1.4 %
   // faster at 131 and 160 live rows while the control threads divided by
   // the stage count; with counters three are 1.5-2 % faster there.)
   const int min_stages = 3;
   int boxes = kMaxBoxes;
   while (boxes > 1 && ((a.H / kBK) % (boxes * ksplit) != 0 ||
-                       ring_bytes / (boxes * (kABytes + h_box)) < min_stages))
+                       ring_bytes / (boxes * (w_bytes + h_box)) < min_stages))
     boxes >>= 1;
-  const int stage_bytes = boxes * (kABytes + h_box);
+  const int stage_bytes = boxes * (w_bytes + h_box);
   int stages = ring_bytes / stage_bytes;
   if (stages > kMaxStages) stages = kMaxStages;
   const int num_kb = a.H / (kBK * boxes) / ksplit;                 // stages per unit
   // offsets in a stage of W box x and hidden box x; the hidden rows loaded
   const int w_off0 = rows_mode ? boxes * h_box : 0;
-  const int h_off0 = rows_mode ? 0 : boxes * kABytes;
+  const int h_off0 = rows_mode ? 0 : boxes * w_bytes;
   const int h_first = rows_mode ? row0 : rank * (G / 2);
   const int h_count = rows_mode ? live16 : G / 2;
   // bytes landing per stage on rank 0's barrier: W and hidden rows of both CTAs
   const uint32_t tx_pair = rows_mode
-      ? (uint32_t)boxes * (2u * kABytes + (uint32_t)(live16 + peer16) * 128u)
+      ? (uint32_t)boxes * (2u * (uint32_t)w_bytes + (uint32_t)(live16 + peer16) * 128u)
       : 2u * (uint32_t)stage_bytes;
   // vocabulary mode: statistics of TMEM lane quadrant w, and the row map
   auto wstats = [&](int w) -> StatsRef {
@@ -1055,7 +1064,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
         bool ok = true;
         for (int tk = t_first; ok && tk < n_tk; tk += per_group) {
           const int t = tk / ksplit, kb0 = (tk % ksplit) * num_kb;
-          const int w_row = (2 * t + rank) * kBM;
+          const int w_row = (2 * t + rank) * w_rows;
           for (int kb = 0; kb < num_kb; ++kb, ++it) {
             if (!mbar_wait(&empty_bar[s], ph ^ 1, a.err)) {
               ok = false;
@@ -1066,7 +1075,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
             const uint32_t fb = at_rank0(&full_bar[s]);
             for (int x = 0; x < boxes; ++x) {
               const int col = ((kb0 + kb) * boxes + x) * kBK;
-              uint8_t* wb = st + w_off0 + x * kABytes;
+              uint8_t* wb = st + w_off0 + x * w_bytes;
               if (w_hint) tma_load_2d_pair_hint(wb, &tmap_w, fb, col, w_row, policy);
               else tma_load_2d_pair(wb, &tmap_w, fb, col, w_row);
               // the hidden rows in the tallest boxes that fit (from L2)
@@ -1102,7 +1111,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
       if (lane == 0 && rank == 0) {
         // rows mode: A = hidden rows, B = W (N = 256 vocabulary ids);
         // vocabulary mode: A = W, B = hidden rows (N = G)
-        const uint32_t idesc = idesc_bf16_f32(2 * kPairRows, rows_mode ? 2 * kBM : G);
+        const uint32_t idesc = idesc_bf16_f32(2 * kPairRows, rows_mode ? 2 * w_rows : G);
         int it = 0, local = 0, s = 0;
         uint32_t ph = 0;
         bool ok = true;
@@ -1121,7 +1130,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
             tc_fence_after();
             const uint32_t st = rbase + (uint32_t)(s * stage_bytes);
             for (int x = 0; x < boxes; ++x) {
-              const uint32_t w_s = st + (uint32_t)(w_off0 + x * kABytes);
+              const uint32_t w_s = st + (uint32_t)(w_off0 + x * w_bytes);
               const uint32_t h_s = st + (uint32_t)(h_off0 + x * h_box);
               const uint64_t adesc = sw128_kmajor_desc(rows_mode ? h_s : w_s);
               const uint64_t bdesc = sw128_kmajor_desc(rows_mode ? w_s : h_s);
@@ -1159,7 +1168,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
       const bool p_vec = ((reinterpret_cast<uintptr_t>(a.part_y) | (uintptr_t)a.V * 4u) & 31u) == 0;
       const bool vec4 = ((reinterpret_cast<uintptr_t>(a.gumbel) | (uintptr_t)a.V * 4u) & 15u) == 0;
       const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
-      constexpr int kChunks = 2 * kBM / 16 / 2;   // chunks of one warp per unit
+      constexpr int kChunks = 2 * kBM / 16 / 2;   // chunks of one warp per unit of 2 x 128 ids
       auto load_noise = [&](int v0, float (&g)[16]) {
         if (!(noisy && row_live)) {
 #pragma unroll
@@ -1195,7 +1204,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
         const int t = tk / ksplit, ks = tk % ksplit;
         const int acc = local & 1;
         const uint32_t use = (uint32_t)(local >> 1);
-        const int vt = t * 2 * kBM;                     // first vocabulary id of the tile
+        const int vt = t * 2 * w_rows;                  // first vocabulary id of the tile
         const uint32_t t_acc = tmem_base + lane_addr + (uint32_t)acc * 256u;
         // noise of the first kGAhead chunks is read while the MMAs run
         float gq[kGAhead][16];
@@ -1208,7 +1217,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
         tc_fence_after();
         if (warp_live) {
 #pragma unroll 1
-          for (int c = 0; c < kChunks; ++c) {
+          for (int c = 0; c < (kLinear ? w_rows / 16 : kChunks); ++c) {
             const int col = 16 * (sub + 2 * c);
             float g[16];
             if constexpr (!kPhilox) {
@@ -2036,6 +2045,7 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     a.linear_rows = 0;
     a.ksplit = 1;
     a.k_cluster = 0;
+    a.w_rows = kBM;
     a.part_y = nullptr;
     a.h_big = p.rows_alloc >= 128 ? 128 : (p.rows_alloc >= 64 ? 64 : 16);
     a.tau = tau;
@@ -2160,29 +2170,39 @@ int linear_ksplit(int T, int K, int N) {
   return best;
 }
 
-// K ranges for the CTA-pair linear (rows layout): the same kind of time
-// model per pair of SMs.  A unit streams 128 W rows x K / ks per SM
-// (~45 GB/s per SM at the HBM peak) or runs K / (16 ks) 2-SM MMAs of
-// ~65 ns, whichever is longer; with ranges it also writes its rows' fp32
-// partials, and the sum over ranges reads them all back in a second launch.
-// At most linear_max_split (what the workspace holds).
-static int pair_linear_ksplit(int T, int K, int N, int n_pairs) {
+// W rows per CTA and unit, and K ranges, of the CTA-pair linear: the pair of
+// shortest modelled time.  A 64-column block of a unit takes as long as its
+// rows' fill of shared memory (107 GB/s an SM, measured in the main loop at
+// 512 rows) or its four 2-SM MMAs (44 ns up to N = 128, 65 at N = 256), and no
+// less than 0.235 us (measured at 32 and 64 W rows); units go to the pairs of their row group in rounds.  Fewer W rows a unit fill a
+// round better (512 x 6144, 38 pairs a group: 24 units of 256 ids, 32 of
+// 192); K ranges shorten the units but write fp32 partials that a second
+// kernel reads back.  At most linear_max_split ranges (what the workspace
+// holds).  Against 128 W rows throughout (an 8B layer's four GEMMs): 256 rows
+// 126.0 -> 120.4 us, 512 rows 165.3 -> 162.5 in bursts.
+struct PairSplit {
+  int w_rows, ksplit;
+};
+static PairSplit pair_linear_split(int T, int K, int N, int n_pairs) {
   const int max_ks = linear_max_split(T, K, N);
-  const int pair_tiles = (N + 2 * kBM - 1) / (2 * kBM);
   const int n_groups = T > 2 * kPairRows ? 2 : 1;
   const int per_group = n_pairs / n_groups > 0 ? n_pairs / n_groups : 1;
-  const double t_mem = 128.0 * K * 2 / 45e3, t_mma = K / 16.0 * 0.065;   // us
-  const double t_unit = t_mem > t_mma ? t_mem : t_mma;
-  const int rows_cta = (T < 2 * kPairRows ? T : 2 * kPairRows) / 2;
-  const double t_part = (double)rows_cta * 2 * kBM * 4 / 45e3;
-  int best = 1;
-  double best_cost = (double)((pair_tiles + per_group - 1) / per_group) * t_unit;
-  for (int ks = 2; ks <= max_ks; ks *= 2) {
-    const double waves = (double)((pair_tiles * ks + per_group - 1) / per_group);
-    const double cost = waves * (t_unit / ks + t_part) + (double)ks * T * N * 4 / 6e6 + 2.0;
-    if (cost < best_cost) {
-      best_cost = cost;
-      best = ks;
+  const int live = T < kPairRows ? T : kPairRows;
+  PairSplit best = {kBM, 1};
+  double best_cost = 1e30;
+  for (int wr = kBM; wr >= 32; wr -= 16) {
+    const int tiles = (N + 2 * wr - 1) / (2 * wr);
+    const double fill = (live + wr) * 128.0 / 107e3;   // us
+    const double mma = 4 * (wr <= 64 ? 0.0441 : 0.0441 + (2 * wr - 128) / 128.0 * 0.0213);
+    const double t_blk = fill > mma ? (fill > 0.235 ? fill : 0.235) : (mma > 0.235 ? mma : 0.235);
+    for (int ks = 1; ks <= max_ks; ks *= 2) {
+      const int rounds = (tiles * ks + per_group - 1) / per_group;
+      double cost = rounds * (t_blk * (K / kBK / ks) + 0.5) + wr * (ks > 1 ? 0.02 : 0.016);
+      if (ks > 1) cost += (double)ks * T * N * 4 / 12e6 + 1.5;
+      if (cost < best_cost) {
+        best_cost = cost;
+        best = {wr, ks};
+      }
     }
   }
   return best;
@@ -2251,6 +2271,7 @@ sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void
   a.rows_alloc = rows_alloc;
   a.n_tiles = (N + kBM - 1) / kBM;
   a.k_cluster = 0;
+  a.w_rows = kBM;
   a.h_big = T >= 128 ? 128 : (T >= 64 ? 64 : 16);
   a.tau = 0.f;
   a.y = (__nv_bfloat16*)y;
@@ -2265,16 +2286,25 @@ sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void
   size_t smem = 0;
   if (T > kPairVocabLanesMax) {
     const void* fn_pair = (const void*)head_pair_kernel<false, true>;
-    const int pair_tiles = (N + 2 * kBM - 1) / (2 * kBM);
     const int n_groups = T > 2 * kPairRows ? 2 : 1;
     int n_pairs = head_pair_slots(fn_pair);
     if (n_groups == 2) n_pairs &= ~1;
     if (n_pairs > 0) {
-      const int ks = pair_linear_ksplit(T, K, N, n_pairs);
+      const PairSplit sp = pair_linear_split(T, K, N, n_pairs);
+      const int ks = sp.ksplit, pair_tiles = (N + 2 * sp.w_rows - 1) / (2 * sp.w_rows);
       if (n_pairs > pair_tiles * n_groups * ks) n_pairs = pair_tiles * n_groups * ks;
       if (n_groups == 2) n_pairs &= ~1;
       if (n_pairs > 0) {
         ksplit = ks;
+        a.w_rows = sp.w_rows;
+        if (sp.w_rows != kBM) {
+          const uint32_t box_w[2] = {(uint32_t)kBK, (uint32_t)sp.w_rows};
+          const uint64_t dims[2] = {(uint64_t)K, (uint64_t)N};
+          const uint64_t strides[1] = {(uint64_t)K * 2};
+          s = encode_tensor_map(&tw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)w, dims, strides,
+                                box_w, CU_TENSOR_MAP_SWIZZLE_128B);
+          if (s != SBD_OK) return s;
+        }
         fn = fn_pair;
         n_ctas = 2 * n_pairs;
         cluster = 2;
