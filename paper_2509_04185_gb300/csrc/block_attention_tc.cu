@@ -220,54 +220,97 @@ struct TcArgs {
   float scale_log2;
 };
 
+// Half `sub` of packed row `row` of Q (zeros past M), on its way from global
+// memory to the swizzled Q tile.  attn_wide_kernel loads it before the block
+// barrier: the producers start behind that barrier and put ~190 KB a CTA into
+// the memory system's queues, and Q loads issued with them came back behind
+// them (barrier to Q ready 5.4 us with 128 CTAs; 128 rows at batch 16, 8192
+// keys 90.8 -> 90.1 us).  attn_tc_kernel has half as many rows and measured
+// 1 % slower that way on ragged batches; it loads after the barrier.
+template <int D>
+struct QHalf {
+  static constexpr int kN = D / 16;            // 16-byte chunks of half a row
+  uint4 v[kN];
+  __device__ __forceinline__ void load(const TcArgs& a, int b, int hkv, int row, int sub) {
+    const __nv_bfloat16* q =
+        a.q + (((size_t)b * a.k + row / a.G) * a.Hq + hkv * a.G + row % a.G) * D + sub * (D / 2);
+#pragma unroll
+    for (int e = 0; e < kN; ++e) v[e] = make_uint4(0, 0, 0, 0);
+    if (row < a.M) {
+#pragma unroll
+      for (int e = 0; e < kN; ++e) v[e] = *reinterpret_cast<const uint4*>(q + e * 8);
+    }
+  }
+  // row `lane_t` of the Q tile at q_s (sub-tiles of 64 columns, kRows x 128 B)
+  __device__ __forceinline__ void store(uint32_t q_s, int lane_t, int sub) const {
+#pragma unroll
+    for (int e = 0; e < kN; ++e) {
+      const int c = sub * kN + e;
+      st_shared_v4(swz(q_s + (c / 8) * (kRows * 128), lane_t, c % 8), v[e]);
+    }
+  }
+};
+
 // ------------------------------------------------ merge in the cluster
 // The CTAs of a cluster are the splits of one (sequence, KV head), each
 // holding its normalised partial rows (cpart_s: kRows x (D + 4) floats) and
 // their log2-sum-exps (after them) in shared memory.  After a cluster
 // barrier every CTA's partials are visible to the others; CTA `rank` merges
-// rows rank, rank + S, ... (softmax warp sw takes one row at a time, lane s
-// reading split s's log2-sum-exp, D / 32 columns a lane) and writes them
-// out; a second barrier keeps every CTA's shared memory alive until the
-// others have read it.  All threads of every CTA reach both barriers: no
-// role leaves the kernel early, and every wait before them is bounded.
-template <int D>
-__device__ __forceinline__ void cluster_merge(const TcArgs& a, int b, int hkv, uint32_t cpart_s,
-                                              int sw, int lane) {
-  cluster_sync_all();
-  if (sw >= 0 && sw < kSoftWarps) {
-    constexpr int kCStride = D + 4;
-    constexpr int kPer = D / 32;
-    const uint32_t clse_s = cpart_s + (uint32_t)(kRows * kCStride * 4);
-    const int S = a.splits;
-    const int rank = (int)cluster_ctarank();
-    for (int r = rank + S * sw; r < a.M; r += S * kSoftWarps) {
-      const float l = lane < S ? ld_cluster_f32(mapa_shared(clse_s + 4u * r, lane)) : -INFINITY;
-      const float gm = warp_max(l);
-      const float w = (lane < S && gm != -INFINITY) ? exp2f(l - gm) : 0.f;
-      const float wsum = warp_sum(w);
-      float v[16][kPer];
+// rows rank, rank + S, ...: a softmax warp takes U rows at a time (U such
+// that U x S partial rows fill its registers), lane s reading split s's
+// log2-sum-exps, D / 32 columns a lane, with every remote read of the U rows
+// requested before the first is used (one row at a time, its sums before its
+// columns, took ~1 us a row: 8 us for 128 rows in clusters of 2).  A second
+// barrier keeps every CTA's shared memory alive until the others have read
+// it.  All threads of every CTA reach both barriers: no role leaves the
+// kernel early, and every wait before them is bounded.
+template <int D, int kS, int kU>
+__device__ __forceinline__ void merge_rows(const TcArgs& a, int b, int hkv, uint32_t cpart_s,
+                                           int rank, int sw, int lane) {
+  constexpr int kCStride = D + 4;
+  constexpr int kPer = D / 32;
+  const uint32_t clse_s = cpart_s + (uint32_t)(kRows * kCStride * 4);
+  const int S = a.splits;
+  const int step = S * kSoftWarps;
+  for (int r0 = rank + S * sw; r0 < a.M; r0 += kU * step) {
+    float l[kU];
+    float v[kU][kS][kPer];
 #pragma unroll
-      for (int s2 = 0; s2 < 16; ++s2) {
-        if (s2 < S) {
-          const uint32_t src = mapa_shared(cpart_s + 4u * (r * kCStride + kPer * lane), s2);
+    for (int u = 0; u < kU; ++u)
+      l[u] = lane < S && r0 + u * step < a.M
+                 ? ld_cluster_f32(mapa_shared(clse_s + 4u * (r0 + u * step), lane)) : -INFINITY;
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+#pragma unroll
+      for (int s2 = 0; s2 < kS; ++s2) {
+        if (s2 < S && r0 + u * step < a.M) {
+          const uint32_t src =
+              mapa_shared(cpart_s + 4u * ((r0 + u * step) * kCStride + kPer * lane), s2);
           if constexpr (kPer == 4) {
             const float4 x = ld_cluster_v4(src);
-            v[s2][0] = x.x; v[s2][1] = x.y; v[s2][2] = x.z; v[s2][3] = x.w;
+            v[u][s2][0] = x.x; v[u][s2][1] = x.y; v[u][s2][2] = x.z; v[u][s2][3] = x.w;
           } else {
             const float2 x = ld_cluster_v2(src);
-            v[s2][0] = x.x; v[s2][1] = x.y;
+            v[u][s2][0] = x.x; v[u][s2][1] = x.y;
           }
         }
       }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int r = r0 + u * step;
+      if (r >= a.M) break;
+      const float gm = warp_max(l[u]);
+      const float w = (lane < S && gm != -INFINITY) ? exp2f(l[u] - gm) : 0.f;
+      const float wsum = warp_sum(w);
       float acc[kPer];
 #pragma unroll
       for (int c = 0; c < kPer; ++c) acc[c] = 0.f;
 #pragma unroll
-      for (int s2 = 0; s2 < 16; ++s2) {
+      for (int s2 = 0; s2 < kS; ++s2) {
         const float ws = __shfl_sync(0xffffffffu, w, s2);    // 0 past S
         if (s2 < S && ws > 0.f) {
 #pragma unroll
-          for (int c = 0; c < kPer; ++c) acc[c] = fmaf(ws, v[s2][c], acc[c]);
+          for (int c = 0; c < kPer; ++c) acc[c] = fmaf(ws, v[u][s2][c], acc[c]);
         }
       }
       const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
@@ -282,6 +325,23 @@ __device__ __forceinline__ void cluster_merge(const TcArgs& a, int b, int hkv, u
         *reinterpret_cast<uint32_t*>(dst) = pack_bf16(acc[0] * inv, acc[1] * inv);
       }
     }
+  }
+}
+
+// (Head dimension 64 takes its rows one at a time: the other forms inlined
+// there cost that kernel's main loop 1.5 %; a call instead of inlining, 1-2 us
+// of every launch.)
+template <int D>
+__device__ __forceinline__ void cluster_merge(const TcArgs& a, int b, int hkv, uint32_t cpart_s,
+                                              int sw, int lane) {
+  cluster_sync_all();
+  if (sw >= 0 && sw < kSoftWarps) {
+    const int rank = (int)cluster_ctarank();
+    if (D == 64) merge_rows<D, 16, 1>(a, b, hkv, cpart_s, rank, sw, lane);
+    else if (a.splits <= 2) merge_rows<D, 2, 8>(a, b, hkv, cpart_s, rank, sw, lane);
+    else if (a.splits <= 4) merge_rows<D, 4, 4>(a, b, hkv, cpart_s, rank, sw, lane);
+    else if (a.splits <= 8) merge_rows<D, 8, 2>(a, b, hkv, cpart_s, rank, sw, lane);
+    else merge_rows<D, 16, 1>(a, b, hkv, cpart_s, rank, sw, lane);
   }
   cluster_sync_all();
 }
@@ -978,6 +1038,8 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_k,
   }
   const int b = a.order ? b_pick : (int)blockIdx.z;
   if (warp == 1) tc_alloc(&tmem_base_sh, kTmemCols);
+  QHalf<D> qh;
+  if (warp >= 3) qh.load(a, b, hkv, (warp & 3) * 32 + lane, (warp - 3) >> 2);
 
   int len = a.lens[b];
   if (len < 0 || len > a.Lmax) {
@@ -1169,14 +1231,7 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_k,
     // Q row -> shared (swizzled, K-major); each sub-warp copies half a row;
     // padding rows are zero.
     {
-      const __nv_bfloat16* qrow =
-          row < a.M ? a.q + (((size_t)b * a.k + row / a.G) * a.Hq + hkv * a.G + row % a.G) * D
-                    : nullptr;
-#pragma unroll
-      for (int c = sub * (D / 16); c < (sub + 1) * (D / 16); ++c) {
-        const uint4 v = qrow ? *reinterpret_cast<const uint4*>(qrow + c * 8) : make_uint4(0, 0, 0, 0);
-        st_shared_v4(swz(q_s + (c / 8) * kQBytes, row, c % 8), v);
-      }
+      qh.store(q_s, row, sub);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&q_ready);
