@@ -36,6 +36,7 @@
 #include <math.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "philox.cuh"
 #include "sbd_internal.cuh"
@@ -850,23 +851,24 @@ constexpr int kPairRows = 128;                 // hidden rows of one CTA per uni
 constexpr int kPairVocabLanesMax = 160;        // live rows up to which the vocabulary layout runs
 
 // One 16-column chunk of a row's logits z (vocabulary ids v0 .. v0 + 15, valid
-// below V) and Gumbel noise g folded into the running statistics.
-__device__ __forceinline__ void fold_chunk16(RowStats& st, const float (&z)[16],
-                                             const float (&g)[16], float tau, int v0, int V) {
+// below V; kFull: all of them are) folded into the running maximum and sums;
+// returns the chunk's maximum of z log2(e) (-inf when no id is valid).
+template <bool kFull>
+__device__ __forceinline__ float fold_sums16(RowStats& st, const float (&z)[16], int v0, int V) {
   float y[16];
   float mc = -INFINITY;
 #pragma unroll
   for (int j = 0; j < 16; ++j) {
-    y[j] = v0 + j < V ? z[j] * kLog2e : -INFINITY;
+    y[j] = kFull || v0 + j < V ? z[j] * kLog2e : -INFINITY;
     mc = fmaxf(mc, y[j]);
   }
-  if (mc == -INFINITY) return;                  // no valid id in this chunk
+  if (mc == -INFINITY) return mc;               // no valid id in this chunk
   const float m_new = fmaxf(st.m, mc);
   float s_add = 0.f, t_add = 0.f;
 #pragma unroll
   for (int j = 0; j < 16; ++j) {
     // invalid ids: 2^-1000 flushes to 0, and 0 * -1000 adds nothing to T
-    const float d = v0 + j < V ? y[j] - m_new : -1000.f;
+    const float d = kFull || v0 + j < V ? y[j] - m_new : -1000.f;
     const float e = ex2_ftz(d);
     s_add += e;
     t_add = fmaf(e, d, t_add);
@@ -882,13 +884,63 @@ __device__ __forceinline__ void fold_chunk16(RowStats& st, const float (&z)[16],
     st.S = s_add;
   }
   st.m = m_new;
+  return mc;
+}
+
+// The chunk's best Gumbel score z + tau g, noise g read.
+template <bool kFull>
+__device__ __forceinline__ void fold_scores16(RowStats& st, const float (&z)[16],
+                                              const float (&g)[16], float tau, int v0, int V) {
 #pragma unroll
   for (int j = 0; j < 16; ++j) {
     // ids ascend within the chunk: a strict > keeps the lowest id on ties
     const float sc = fmaf(tau, g[j], z[j]);
-    if (v0 + j < V && sc > st.best) {
+    if ((kFull || v0 + j < V) && sc > st.best) {
       st.best = sc;
       st.idx = v0 + j;
+    }
+  }
+}
+
+// The same with the noise still in its random words x[j] (tau > 0; mc the
+// chunk's maximum of z log2(e)).  A score beats st.best only if its noise
+// exceeds d = (best - max z) / tau; the noise of 1 - u = (m + 1/2) 2^-23, with
+// m = ~x >> 9, does so only if 1 - u < -ln u < exp(-d), so one compare a word
+// against a bound shared by the chunk rules out nearly all of them without a
+// logarithm: a row sees a new best about ln n times in n ids.  The others are
+// scored exactly, in ascending order, so the winner is that of scoring every
+// id.  d is lowered by more than the roundings of the noise (1e-5 here), the
+// score (2^-24 of it) and this bound, and every comparison that is not
+// decided (infinite or NaN d) falls on the exact side or cannot win.
+// Per call at V = 128256, H = 4096 (bursts), two logarithms a logit against
+// this: 200 rows 227 -> 205 us, 256 rows 225 -> 210, 320 rows 435 -> 385, 512
+// rows 460 -> 380 (the noise buffer: 203, 209, 346, 351); V = 151936, 512
+// rows, under the power cap 486 -> 450.  Most of the rest are the generator's
+// rounds.  (Round keys from the host made no difference.)
+template <bool kFull>
+__device__ __forceinline__ void fold_words16(RowStats& st, const float (&z)[16],
+                                             const uint32_t (&x)[16], float mc, float tau,
+                                             float inv_tau, int v0, int V) {
+  const float z_max = fmaf(fabsf(mc), 1e-6f, mc * kLn2);
+  const float d = (st.best - z_max) * inv_tau;
+  const float eps =
+      fmaf(fabsf(d), 1e-5f, fmaf(fabsf(st.best) + fabsf(z_max), 1e-6f * inv_tau, 5e-5f));
+  // exp(-(d - eps)) 2^23, rounded up; above 2^23 every word qualifies
+  const float bound = fmaf(ex2_ftz((eps - d) * kLog2e), 8388608.f * 1.0001f, 1.f);
+  const uint32_t t = bound < 8388608.f ? (uint32_t)bound + 1u : 8388608u;   // m < t qualifies
+  const uint32_t x_min = 0u - (t << 9);          // ~x >> 9 < t; 0 when t = 2^23
+  uint32_t x_top = 0u;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) x_top = max(x_top, x[j]);
+  if (x_top < x_min) return;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    if (x[j] >= x_min && (kFull || v0 + j < V)) {
+      const float sc = fmaf(tau, sbd_philox::gumbel_of_word(x[j]), z[j]);
+      if (sc > st.best) {
+        st.best = sc;
+        st.idx = v0 + j;
+      }
     }
   }
 }
@@ -1173,16 +1225,6 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
         if (!(noisy && row_live)) {
 #pragma unroll
           for (int j = 0; j < 16; ++j) g[j] = 0.f;
-        } else if constexpr (kPhilox) {
-          // one call gives the words of ids 4q .. 4q + 3 (v0 is a multiple of 16)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const uint4 x = sbd_philox::philox4x32_10(
-                make_uint4(((uint32_t)v0 >> 2) + (uint32_t)i, (uint32_t)n, a.off_lo, a.off_hi),
-                a.seed_lo, a.seed_hi);
-#pragma unroll
-            for (int w = 0; w < 4; ++w) g[4 * i + w] = sbd_philox::gumbel_of_word(sbd_philox::word_of(x, w));
-          }
         } else if (vec4) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -1199,6 +1241,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
         }
       };
       RowStats st = rowstats_empty();
+      const float inv_tau = 1.f / a.tau;
       int local = 0;
       for (int tk = t_first; tk < n_tk; tk += per_group, ++local) {
         const int t = tk / ksplit, ks = tk % ksplit;
@@ -1228,8 +1271,21 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
 #pragma unroll
                 for (int j = 0; j < 16; ++j) gq[d][j] = gq[d + 1][j];
               if (c + kGAhead < kChunks) load_noise(vt + col + 32 * kGAhead, gq[kGAhead - 1]);
-            } else {
-              load_noise(vt + col, g);
+            }
+            uint32_t words[16];
+            if constexpr (kPhilox) {
+              // one call gives the words of ids 4q .. 4q + 3 (col is a multiple
+              // of 16); made while the accumulators are on their way
+              if (noisy && row_live) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const uint4 x = sbd_philox::philox4x32_10(
+                      make_uint4(((uint32_t)(vt + col) >> 2) + (uint32_t)i, (uint32_t)n, a.off_lo, a.off_hi),
+                      a.seed_lo, a.seed_hi);
+#pragma unroll
+                  for (int w = 0; w < 4; ++w) words[4 * i + w] = sbd_philox::word_of(x, w);
+                }
+              }
             }
             uint32_t r[16];
             tc_ld_32x32b_x16(t_acc + (uint32_t)col, r);
@@ -1271,7 +1327,23 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
                   }
                 }
               } else {
-                fold_chunk16(st, z, g, a.tau, vt + col, a.V);
+                const int v0 = vt + col;
+                auto fold = [&](auto full) {
+                  constexpr bool kFull = decltype(full)::value;
+                  const float mc = fold_sums16<kFull>(st, z, v0, a.V);
+                  if (kPhilox && noisy) {
+                    if (mc != -INFINITY)
+                      fold_words16<kFull>(st, z, words, mc, a.tau, inv_tau, v0, a.V);
+                  } else {
+                    if constexpr (kPhilox) {
+#pragma unroll
+                      for (int j = 0; j < 16; ++j) g[j] = 0.f;
+                    }
+                    fold_scores16<kFull>(st, z, g, a.tau, v0, a.V);
+                  }
+                };
+                if (v0 + 16 <= a.V) fold(std::true_type{});
+                else fold(std::false_type{});
               }
             }
           }

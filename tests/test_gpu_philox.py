@@ -107,3 +107,25 @@ def test_fresh_offsets_give_fresh_samples(sbd):
     assert any(not np.array_equal(toks[0], x) for x in toks[1:])
     again = sbd.sbd_head_entropy_sample_philox(hid, W, m, 7, 0, 1.0)[1].cpu().numpy()
     assert np.array_equal(toks[0], again)                       # same counter, same sample
+
+
+@pytest.mark.parametrize("tau", [1e-35, 1e-3, 1.0, 40.0])
+@pytest.mark.parametrize("scale", [0.0, 1e-3, 1.0, 300.0])
+def test_rows_layout_scores_every_id_that_can_win(sbd, tau, scale):
+    """Above 160 rows the in-kernel noise is turned into a score only where its
+    random word can beat the best so far: the winner must be that of scoring
+    every id (the same noise from a buffer), bit for bit, for logits that are
+    all equal, small, ordinary and huge, weak and strong noise, and a
+    vocabulary that ends inside a 16-id chunk."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(3)
+    B, k, H, V = 12, 16, 128, 9001
+    hid = (torch.randn(B, k, H, generator=g, device="cuda") * scale).to(torch.bfloat16)
+    w = torch.randn(V, H, generator=g, device="cuda").to(torch.bfloat16)
+    masked = torch.ones(B, k, dtype=torch.uint8, device="cuda")
+    ids = torch.arange(B * k, dtype=torch.int32, device="cuda")
+    noise = sbd.sbd_gumbel_philox(ids, V, 77, 11).view(B, k, V)
+    e1, t1 = sbd.sbd_head_entropy_sample_philox(hid, w, masked, 77, 11, tau)
+    e2, t2 = sbd.sbd_head_entropy_sample(hid, w, masked, noise, tau)
+    assert torch.equal(t1, t2) and torch.equal(e1, e2)
+    assert sbd.sbd_device_error() == 0
