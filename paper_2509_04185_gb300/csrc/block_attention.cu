@@ -505,6 +505,7 @@ AttnPlan attn_plan(const sbd_attn_desc& d) {
   } else {
     p.splits = choose_splits(p.B * p.Hkv, tiles, num_sms());
   }
+  p.wide = p.bf16 && attn_use_wide(p);
   // tcgen05 path: the splits of a (sequence, KV head) merge in shared memory
   // as one thread-block cluster (at most 16 CTAs) when the device can hold
   // all the clusters at once.  An automatic split count is lowered, down to

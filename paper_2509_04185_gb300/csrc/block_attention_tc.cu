@@ -37,8 +37,6 @@
 // (one split) or the split partial and its log-sum-exp.
 #include <math.h>
 
-#include <mutex>
-
 #include "sbd_internal.cuh"
 
 namespace {
@@ -1444,56 +1442,41 @@ static size_t attn_wide_smem_bytes(int D) {
          (size_t)v_slots * sub * kTileKeys * 128;
 }
 
-// The kernel for head dimension D and M packed rows: up to 64 rows
-// attn_tc_kernel with every row copied into both lane halves, above that
-// attn_wide_kernel.
+// The kernel of plan p: attn_wide_kernel, or attn_tc_kernel with every row
+// copied into both lane halves (up to 64 packed rows; see attn_use_wide).
 struct TcKernel {
   const void* fn;
   int threads;
   size_t smem;
 };
-static TcKernel attn_tc_kernel_for(int D, int M) {
-  if (M <= kRows / 2)
-    return TcKernel{D == 128 ? (const void*)attn_tc_kernel<128, 2> : (const void*)attn_tc_kernel<64, 2>,
-                    kThreads, attn_tc_smem_bytes(D)};
-  return TcKernel{D == 128 ? (const void*)attn_wide_kernel<128> : (const void*)attn_wide_kernel<64>,
-                  kWideThreads, attn_wide_smem_bytes(D)};
+static TcKernel attn_tc_kernel_for(const AttnPlan& p) {
+  if (!p.wide)
+    return TcKernel{p.D == 128 ? (const void*)attn_tc_kernel<128, 2> : (const void*)attn_tc_kernel<64, 2>,
+                    kThreads, attn_tc_smem_bytes(p.D)};
+  return TcKernel{p.D == 128 ? (const void*)attn_wide_kernel<128> : (const void*)attn_wide_kernel<64>,
+                  kWideThreads, attn_wide_smem_bytes(p.D)};
+}
+
+// Above 64 packed rows only attn_wide_kernel serves.  Up to 64, at head
+// dimension 128, it is the faster one where a CTA has few keys (two triples
+// against three pairs: batch 1, 16 rows x 4 heads, 500 / 1000 / 4096 keys
+// 9.9 / 10.5 / 11.9 -> 9.0 / 9.6 / 11.0 us) and where the launch takes several
+// waves (its shared-memory traffic per key is a quarter less: 32 x 2048 keys
+// 57.8 -> 55.8 us, 64 ragged to 2000 81.7 -> 77.9).  attn_tc_kernel's shorter
+// chain of MMAs wins on long ranges of uneven length, where the longest CTA
+// sets the time (batch 4 ragged to 32768 81.0 against 84.6), and at head
+// dimension 64 (batch 16 ragged to 8000 64 against 76).
+bool attn_use_wide(const AttnPlan& p) {
+  if (p.M > kRows / 2) return true;
+  if (p.D != 128) return false;
+  return 2ll * p.B * p.Hkv >= 3ll * num_sms() || p.Lmax <= 256ll * p.splits;
 }
 
 bool attn_tc_cluster_ok(const AttnPlan& p, int splits) {
   // Whether every (sequence, KV head)'s `splits` CTAs can run as one cluster,
-  // all clusters at once.  The device's answer per (device, kernel, cluster
-  // size) is kept; the call is on every launch's host path.
-  struct Entry {
-    int dev;
-    const void* fn;
-    int splits;
-    int clusters;
-  };
-  static std::mutex mu;
-  static Entry cache[32];
-  static int n_cache = 0;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  const TcKernel kern = attn_tc_kernel_for(p.D, p.M);
-  const void* fn = kern.fn;
-  int clusters = -1;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    for (int i = 0; i < n_cache; ++i)
-      if (cache[i].dev == dev && cache[i].fn == fn && cache[i].splits == splits)
-        clusters = cache[i].clusters;
-  }
-  if (clusters < 0) {
-    clusters = max_active_clusters(fn, dim3(splits, p.Hkv, p.B), dim3(kern.threads), kern.smem,
-                                   splits);
-    std::lock_guard<std::mutex> lock(mu);
-    if (n_cache < 32) cache[n_cache++] = Entry{dev, fn, splits, clusters};
-  }
-  return (long long)clusters >= (long long)p.B * p.Hkv;
+  // all clusters at once.
+  const TcKernel kern = attn_tc_kernel_for(p);
+  return (long long)cluster_slots(kern.fn, kern.threads, kern.smem, splits) >= (long long)p.B * p.Hkv;
 }
 
 sbd_status attn_tc_launch(const AttnPlan& p, const CUtensorMap& tk, const CUtensorMap& tv,
@@ -1523,7 +1506,7 @@ sbd_status attn_tc_launch(const AttnPlan& p, const CUtensorMap& tk, const CUtens
   a.vc_app = (__nv_bfloat16*)vc_app;
   a.scale_log2 = p.scale_log2;
   a.cluster = p.cluster ? 1 : 0;
-  const TcKernel kern = attn_tc_kernel_for(p.D, p.M);
+  const TcKernel kern = attn_tc_kernel_for(p);
   const size_t smem = kern.smem;
   const void* fn = kern.fn;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -33,6 +33,7 @@ sbd_status encode_tensor_map(CUtensorMap* map, CUtensorMapDataType dtype, uint32
 struct AttnPlan {
   int B, k, Hq, Hkv, G, D, Lmax, M, splits;
   bool order;         // CTAs take sequences longest first (more than one wave)
+  bool wide;          // bf16: attn_wide_kernel, else attn_tc_kernel
   bool cluster;       // the splits of a (sequence, KV head) merge in a cluster (tcgen05 path)
   int n_causal;       // block rows i < n_causal see block keys j <= i only
   float scale_log2;   // softmax scale * log2(e)
@@ -47,6 +48,8 @@ sbd_status attn_launch(const AttnPlan& p, const void* q, const void* kc, const v
                        void* ws, void* kc_app, void* vc_app, cudaStream_t st);
 
 size_t attn_tc_smem_bytes(int D);
+// Which tcgen05 kernel serves plan p (its shape and split count).
+bool attn_use_wide(const AttnPlan& p);
 // Whether the tcgen05 attention kernel can run the `splits` CTAs of every
 // (sequence, KV head) of plan p as one thread-block cluster, all at once.
 bool attn_tc_cluster_ok(const AttnPlan& p, int splits);

@@ -159,3 +159,20 @@ def test_f32_split_and_tile_edges(sbd, G, k, D, n_causal):
     w = gen.shrink(w, batch=1, cache_len=(0, 2100))
     _check(sbd, w, _inputs(w, G * k + 1, [2081]), n_causal)
     assert sbd.sbd_device_error() == 0
+
+
+@pytest.mark.parametrize("n_causal", [0, 2])
+@pytest.mark.parametrize("splits", [1, 2, 3, 6])
+@pytest.mark.parametrize("G,k", [(1, 2), (4, 4), (3, 11), (4, 16)])
+def test_bf16_both_kernels_up_to_64_rows(sbd, G, k, splits, n_causal):
+    """Head dimension 128, up to 64 packed rows: 256 keys a split and fewer
+    run on the wide kernel, more on the paired one; the same lengths at
+    capacities on both sides of that line."""
+    lens = [0, 1, 63, 64, 65, 191, 192, 256, 257]
+    for cap in (256 * splits, 256 * splits + 1):
+        cap = max(cap, 257 + k)
+        w = gen.shrink(BF16, batch=len(lens), block_k=k, n_q_heads=G, n_kv_heads=1, cache_len=(0, cap))
+        _check(sbd, w, _inputs(w, splits + k, lens), n_causal, num_splits=splits)
+    w = gen.shrink(BF16, batch=2, block_k=k, n_q_heads=2 * G, n_kv_heads=2, cache_len=(0, 1700))
+    _check(sbd, w, _inputs(w, splits + k + 1, [1690, 1025]), n_causal, num_splits=splits)
+    assert sbd.sbd_device_error() == 0
