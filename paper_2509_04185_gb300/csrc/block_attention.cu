@@ -505,7 +505,7 @@ AttnPlan attn_plan(const sbd_attn_desc& d) {
   } else {
     p.splits = choose_splits(p.B * p.Hkv, tiles, num_sms());
   }
-  p.wide = p.bf16 && attn_use_wide(p);
+  p.wide = p.bf16 && p.M > 64;
   // tcgen05 path: the splits of a (sequence, KV head) merge in shared memory
   // as one thread-block cluster (at most 16 CTAs) when the device can hold
   // all the clusters at once.  An automatic split count is lowered, down to
@@ -525,6 +525,12 @@ AttnPlan attn_plan(const sbd_attn_desc& d) {
         break;
       }
     }
+  }
+  // The kernel by the keys of a CTA; both hold the same clusters (one 227 KB
+  // CTA per SM), else the choice stays.
+  if (p.bf16 && !p.wide) {
+    p.wide = attn_use_wide(p);
+    if (p.wide && p.cluster && !attn_tc_cluster_ok(p, p.splits)) p.wide = false;
   }
   // With more CTAs than one wave, the CTAs take the sequences longest first
   // (the pick costs B^2 comparisons per CTA, hence the batch limit).

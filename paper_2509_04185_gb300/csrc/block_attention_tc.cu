@@ -15,26 +15,24 @@
 //                     TMEM.
 //
 // Pairs, not single tiles: an M = 128, K = 16 tcgen05.mma measured about the
-// same time for N = 64, 128 and 256 (~135 cycles), so 64-key score products
-// left the tensor pipe the bottleneck (1300 cycles of MMA per 64 keys; 760
-// with 128-key pairs).  The two tiles of a pair sit back to back in every
-// 128-byte sub-tile of the ring, so that they form one 128-row operand.
+// same time for N = 64 and 128 (47.6 ns; 65.4 at N = 256), so 64-key score
+// products left the tensor pipe the bottleneck.  The two tiles of a pair sit
+// back to back in every 128-byte sub-tile of the ring, so that they form one
+// 128-row operand.
 //
-// Warp roles: warp 0 streams K/V tiles with TMA (a ring of 3 pairs), the k
-// block keys/values included (the last tile of the last split); warp 1
-// owns the tensor memory and one thread issues the MMAs, computing S_{q+1}
-// while the softmax of pair q runs; warps 2-9 are the softmax, two per TMEM
-// lane quadrant (and, with 64 packed rows or fewer, each row copied to a
-// second quadrant, so that four warps share a row): a thread reads its share
-// of a row's 128 scores with tcgen05.ld, applies the mask (cache key < L_b,
-// block key < k, or j <= i for a causal block row i < n_causal) and the
-// scale, and writes its part of P_q = 2^(s - m_ref) as bf16 into shared
-// memory.  The warps sharing a row agree on the pair's row maximum through a
-// shared-memory exchange.  The reference max m_ref only moves (and O is
-// rescaled in tensor memory) when the running max exceeds it by more than
-// 2^8, which keeps every P entry <= 256; l and O use the same reference, so
-// the result is exact.  The epilogue normalises O by l and writes the output
-// (one split) or the split partial and its log-sum-exp.
+// Warp roles: warp 0 streams K/V tiles with TMA (a ring of 3 pairs, 5 at
+// D = 64), the k block keys/values included (the last tile of the last
+// split); warp 1 owns the tensor memory and one thread issues the MMAs, scores
+// up to two pairs ahead; warps 2-9 are the softmax, two groups of four (one
+// warp per TMEM lane quadrant) on alternate pairs: a thread reads its share
+// of a row's scores with tcgen05.ld (each row is copied to a second lane, one
+// per tile of the pair), applies the mask (cache key < L_b, block key < k, or
+// j <= i for a causal block row i < n_causal) and the scale, and writes its
+// part of P_q = 2^(s - m_ref) as bf16 into shared memory.  The reference max
+// m_ref only moves (and O is rescaled in tensor memory) when the running max
+// exceeds it by more than 2^8, which keeps every P entry <= 256; l and O use
+// the same reference, so the result is exact.  The epilogue normalises O by l
+// and writes the output (one split) or the split partial and its log-sum-exp.
 #include <math.h>
 
 #include "sbd_internal.cuh"
@@ -45,7 +43,7 @@ using namespace sbd_dev;
 
 constexpr int kTileKeys = 64;              // keys per TMA stage
 constexpr int kPairKeys = 2 * kTileKeys;   // keys per MMA step (two stages)
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 10;
 constexpr int kMaxPairs = kMaxStages / 2;
 constexpr int kRows = 128;                 // MMA M (packed rows, padded)
 constexpr int kSoftWarps = 8;              // two per TMEM lane quadrant
@@ -344,27 +342,36 @@ __device__ __forceinline__ void cluster_merge(const TcArgs& a, int b, int hkv, u
   cluster_sync_all();
 }
 
-// Softmax work split over the 128 columns of a pair.  R = 1: packed row r
-// lives in TMEM lane r, and the two warps of its lane quadrant take 64 of the
-// pair's 128 columns each (one tile each).  R = 2 (M <= 64): rows are also
-// copied to lanes 64 + r (the MMA pads to 128 rows anyway), so four warps on
-// all four SM sub-partitions share a row, 32 columns each: copy 0 (lanes
-// 0-63) takes the pair's first tile, copy 1 (lanes 64-127) the second.  The
-// warps sharing a row exchange their partial maxima through shared memory at
-// a named barrier and take identical decisions.
+// Every packed row r sits in two TMEM lanes (the MMA pads to 128 rows anyway):
+// copy 0 (lane r) takes a pair's first tile, copy 1 (lane 64 + r) the second.
+// The eight softmax warps form two groups of four, one warp per lane quadrant:
+// group 0 takes the even pairs, group 1 the odd ones, a lane its copy's 64
+// columns of the pair.  A row's 64 scores lie in one thread, so no maximum is
+// exchanged between warps, and the groups' latencies (TMEM read, exponentials,
+// fences) overlap.  With all eight warps on every pair, 32 columns each and an
+// exchange of maxima, and scores one pair ahead, the chain S -> softmax -> P
+// -> PV set the pace where HBM did not: batch 16, head dimension 64, ragged to
+// 8000 keys 64.3 -> 53.2 us; head dimension 128, 16 rows: batch 4, 32768 keys
+// 91.1 -> 87.6, batch 16, 8192 keys 89.7 -> 86.0 (HBM: 79.3, 79.8).  The groups
+// alone were worth 1 %: a group still waited for its next scores, issued only
+// after the other's PV.
 //
-// PV with R = 2.  A tcgen05.mma of M = 128 and K = 16 costs nearly as much
-// at N = 128 as at N = 256 (47.6 against 65.4 ns of throughput on GB300),
-// and the MMAs lie on the chain S -> softmax -> P -> PV, so N = D would pay
-// almost a full instruction for half its work.  Each copy of a row
-// therefore accumulates its own tile only: lane r of P holds the row's
+// Every copy has its own softmax reference and sums, merged in the epilogue.
+// With D = 64 every group also has its own O (2 x 2 D columns of TMEM).  With
+// D = 128 the groups share O and so the reference, which passes from pair to
+// pair, i.e. from group to group, through shared memory, one named barrier per
+// quadrant and pair parity (the writer arrives, the reader waits).
+//
+// PV.  A tcgen05.mma of M = 128 and K = 16 costs nearly as much at N = 128 as
+// at N = 256 (47.6 against 65.4 ns of throughput on GB300), so N = D would pay
+// almost a full instruction for half its work.  Lane r of P holds the row's
 // probabilities over the keys of its copy's tile, and one instruction with
 // B = [V of 16 keys of tile 0 | V of the same 16 rows of tile 1] (N = 2 D)
-// adds P_copy0 V_tile0 to columns
-// [0, D) and P_copy1 V_tile1 to columns [D, 2 D) of O (the other two blocks
-// of the product land in columns no lane reads).  4 instructions per pair
-// instead of 8; the two partial sums of a row are added in the epilogue.
-template <int D, int R>
+// adds P_copy0 V_tile0 to columns [0, D) and P_copy1 V_tile1 to columns
+// [D, 2 D) of O (the other two blocks of the product land in columns no lane
+// reads).  4 instructions per pair instead of 8; the partial sums of a row
+// are added in the epilogue.
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
                const __grid_constant__ CUtensorMap tmap_v,
@@ -375,15 +382,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
   constexpr int kKVSub = kTileKeys * 128;          // one tile's K or V sub-tile: 8 KB
   constexpr int kPairSub = 2 * kKVSub;             // a pair's K or V sub-tile: 16 KB
   constexpr int kPairBytes = 2 * kSub * kPairSub;  // K sub-tiles then V sub-tiles
-  constexpr uint32_t kTmemCols = 512;              // S0 | S1 (128 each) | O (R * D)
+  constexpr uint32_t kTmemCols = 512;              // S0 | S1 (128 each) | O (2 D a set)
   constexpr uint32_t kOCol = 2 * kPairKeys;
-  static_assert(R == 1 || R == 2, "row copies");
-  static_assert(kOCol + R * D <= kTmemCols, "O fits the allocation");
+  constexpr bool kSharedO = D == 128;              // one O for both groups, or one each
+  constexpr int kOSets = kSharedO ? 1 : 2;
+  static_assert(kOCol + kOSets * 2 * D <= kTmemCols, "O fits the allocation");
   // With D = 128 the K region of a pair (32 KB) is exactly a P block, and K is
   // dead once S of the pair is computed: P is written there, and the ring gets
   // the shared memory separate P buffers would take.
   constexpr bool kPInK = D == 128;
-  constexpr int kPairs = kPInK ? 3 : 4;            // ring depth in pairs
+  constexpr int kPairs = kPInK ? 3 : 5;            // ring depth in pairs
   constexpr int kStages = 2 * kPairs;              // ring depth in 64-key tiles
   static_assert(kQBytes == kPairSub, "a P sub-tile fills a pair's K sub-tile");
 
@@ -392,17 +400,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
   __shared__ __align__(8) uint64_t s_full[2], s_free[2], p_full[2], pv_done[2];
   __shared__ __align__(8) uint64_t q_ready, tail_bar;
   __shared__ uint32_t tmem_base_sh;
-  // Exchange buffer of the softmax warps: partial row maxima as bf16 rounded
-  // up ([pair parity][warp][lane]), then, at the end, fp32 partial row sums
-  // ([warp][lane]).  1 KB: the ring and Q take the rest of the 227 KB.
-  __shared__ __align__(16) uint32_t red_buf[kSoftWarps * 32];
-  uint16_t* red_max = reinterpret_cast<uint16_t*>(red_buf);
-  float* red_l = reinterpret_cast<float*>(red_buf);
+  // Per TMEM lane: the softmax reference of every O set, and at the end every
+  // group's sum of probabilities.
+  __shared__ float m_sh[kOSets][kRows], l_sh[2][kRows];
 
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t q_s = sbase;                              // kSub x 16 KB
-  const uint32_t p_s = q_s + kSub * kQBytes;               // 2 x 32 KB unless kPInK
-  const uint32_t kv_s = p_s + (kPInK ? 0 : 4 * kQBytes);   // kPairs x kPairBytes
+  const uint32_t p_s = q_s + kSub * kQBytes;               // 2 x 16 KB unless kPInK
+  const uint32_t kv_s = p_s + (kPInK ? 0 : 2 * kQBytes);   // kPairs x kPairBytes
   // Tile j of this split lives in pair slot (j / 2) mod kPairs, half j mod 2.
   // K: the two tiles of a pair sit back to back in every sub-tile, so that a
   // pair's keys form one 128-row operand of S.  V: the sub-tiles are ordered
@@ -415,10 +420,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
   auto v_chunk = [&](int j, int h) -> uint32_t {
     return kv_s + ((j >> 1) % kPairs) * kPairBytes + kSub * kPairSub + ((j & 1) * kSub + h) * kKVSub;
   };
-  // P block of pair q: R = 1, two 16 KB sub-tiles (keys 0-63, 64-127); R = 2,
-  // one sub-tile whose row r holds lane r's keys (its copy's tile)
+  // P block of pair q: one 16 KB sub-tile whose row r holds lane r's keys (its
+  // copy's tile)
   auto p_block = [&](int q) -> uint32_t {
-    return kPInK ? k_chunk(2 * q, 0) : p_s + (q & 1) * 2 * kQBytes;
+    return kPInK ? k_chunk(2 * q, 0) : p_s + (q & 1) * kQBytes;
   };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -430,8 +435,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     for (int s = 0; s < kPairs; ++s) mbar_init(&kv_empty[s], 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&s_free[i], kSoftWarps);      // one arrival per softmax warp
-      mbar_init(&p_full[i], kSoftWarps);
+      mbar_init(&s_free[i], kSoftWarps / 2);  // one arrival per warp of the pair's group
+      mbar_init(&p_full[i], kSoftWarps / 2);
       mbar_init(&pv_done[i], 1);
     }
     mbar_init(&q_ready, kSoftWarps);
@@ -563,7 +568,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     if (lane == 0 && n > 0) {
-      const uint32_t id_o = idesc_bf16(kRows, D, true);
       bool ok = mbar_wait(&q_ready, 0, a.err);
       tc_fence_after();
       // S of pair q: M = 128 rows, N = 128 keys (64 for a last single tile),
@@ -581,83 +585,77 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
         }
         tc_commit(&s_full[q & 1]);
       };
-      // O += P V over the pair's keys, 16 keys per instruction (R = 1), or
-      // 16 keys of each tile per instruction into the two copies' halves of
-      // O (R = 2; N = D only for a last pair of one tile, whose second copy
-      // has no keys).
+      // O += P V over the pair's keys: 16 keys of each tile per instruction into
+      // the two copies' halves of O (N = D only for a last pair of one tile,
+      // whose second copy has no keys).
       auto issue_pv = [&](int q) {
         const int nt = min(2, n - 2 * q);
         const uint32_t pb = p_block(q);
         const uint32_t vb = v_chunk(2 * q, 0);
-        if constexpr (R == 1) {
+        const uint32_t o = tmem + kOCol + (kSharedO ? 0u : (uint32_t)((q & 1) * 2 * D));
+        const bool begun = q >= kOSets;              // the O set holds a sum already
+        const uint32_t id_pv = idesc_bf16(kRows, nt * D, true);
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            if (kk >= 4 * nt) break;
-            const uint64_t ad = sw128_desc(pb + (kk / 4) * kQBytes + (kk % 4) * 32, 16, 1024);
-            const uint64_t bd = sw128_desc(vb + (kk / 4) * kSub * kKVSub + (kk % 4) * 16 * 128,
-                                           kKVSub, 1024);
-            tc_mma(tmem + kOCol, ad, bd, id_o, (q > 0 || kk > 0) ? 1u : 0u);
-          }
-        } else {
-          const uint32_t id_pv = idesc_bf16(kRows, nt * D, true);
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t ad = sw128_desc(pb + kk * 32, 16, 1024);
-            const uint64_t bd = sw128_desc(vb + kk * 16 * 128, kKVSub, 1024);
-            tc_mma(tmem + kOCol, ad, bd, id_pv, (q > 0 || kk > 0) ? 1u : 0u);
-          }
+        for (int kk = 0; kk < 4; ++kk) {
+          const uint64_t ad = sw128_desc(pb + kk * 32, 16, 1024);
+          const uint64_t bd = sw128_desc(vb + kk * 16 * 128, kKVSub, 1024);
+          tc_mma(o, ad, bd, id_pv, (begun || kk > 0) ? 1u : 0u);
         }
         tc_commit(&pv_done[q & 1]);
         tc_commit(&kv_empty[q % kPairs]);
       };
-      // In order: S_{q+1} is issued before waiting for P_q, so the scores of
-      // the next pair are computed while the softmax of this one runs; and
-      // since S_{q+1} is issued after PV_{q-1}, the completion of S_{q+1}
-      // (s_full) implies PV_{q-1} is done, which keeps every later parity
-      // wait on pv_done at most one phase behind.
-      auto wait_issue_s = [&](int q) -> bool {
-        const int j0 = 2 * q, nt = min(2, n - j0);
-        for (int e = 0; e < nt; ++e)
-          if (!mbar_wait(&kv_full[(j0 + e) % kStages], ((j0 + e) / kStages) & 1, a.err)) return false;
-        if (!mbar_wait(&s_free[q & 1], ((q >> 1) & 1) ^ 1, a.err)) return false;
-        tc_fence_after();
-        issue_s(q);
-        return true;
-      };
-      if (ok) ok = wait_issue_s(0);
-      // (Issuing PV_q ahead of S_{q+1} when P_q is ready first measured
-      // slower: the next softmax then waits longer for its scores.)
-      for (int q = 0; q < np && ok; ++q) {
-        if (q + 1 < np && !wait_issue_s(q + 1)) break;
-        if (!mbar_wait(&p_full[q & 1], (q >> 1) & 1, a.err)) break;
-        tc_fence_after();
-        issue_pv(q);
+      // Scores run up to two pairs ahead: S_{q+2} goes out as soon as its keys
+      // are there and group q mod 2 has read S_q, usually before P_q is ready,
+      // so that a group that hands in its P finds its next scores done; PV_q
+      // goes out when P_q is there.  Whichever is ready first is issued, S_s
+      // never before PV_{s-3}: s_full of S_q implies that PV_{q-3} is done,
+      // and a group waits for PV_{q-2} before it hands in P_q, so every parity
+      // wait on pv_done is at most one phase behind.
+      int next_s = 0, next_pv = 0;
+      uint64_t t0 = 0;
+      for (uint32_t idle = 0; ok && next_pv < np;) {
+        bool moved = false;
+        if (next_s < np && next_s <= next_pv + 2) {
+          const int j0 = 2 * next_s, j1 = j0 + min(2, n - j0) - 1;
+          if (mbar_poll_parity(&kv_full[j0 % kStages], (j0 / kStages) & 1) &&
+              mbar_poll_parity(&kv_full[j1 % kStages], (j1 / kStages) & 1) &&
+              mbar_poll_parity(&s_free[next_s & 1], ((next_s >> 1) & 1) ^ 1)) {
+            tc_fence_after();
+            issue_s(next_s++);
+            moved = true;
+          }
+        }
+        if (next_pv < next_s && mbar_poll_parity(&p_full[next_pv & 1], (next_pv >> 1) & 1)) {
+          tc_fence_after();
+          issue_pv(next_pv++);
+          moved = true;
+        }
+        if (moved) {
+          idle = 0;
+        } else if ((++idle & 63u) == 0) {            // bounded, as mbar_wait
+          const uint64_t now = globaltimer();
+          if (idle == 64) t0 = now;
+          if (now - t0 > kWaitLimitNs) {
+            record_error(a.err, SBD_DEVERR_TIMEOUT);
+            ok = false;
+          }
+        }
       }
     }
   } else {
     // ------------------------------------------------ softmax warps
-    constexpr int kCW = kPairKeys / (2 * R);     // columns per warp: 64 or 32
-    constexpr int kQuadStride = 4 / R;           // lane quadrants between copies of a row
-    constexpr int kRowsPerCopy = kRows / R;
-    constexpr int kGroupThreads = 64 * R;        // the warps that share a row
+    constexpr int kCW = kTileKeys;               // columns per lane: its copy's tile
     const int sw = warp - 2;                     // 0..7
     const int quad = warp & 3;                   // TMEM lanes 32*quad .. +31
-    const int sub = sw >> 2;                     // 0 or 1 within the quadrant
+    const int sub = sw >> 2;                     // the warp's group: pairs sub, sub + 2, ...
     const int lane_t = quad * 32 + lane;         // TMEM lane
-    const int row = lane_t % kRowsPerCopy;       // packed row
-    const int dup = lane_t / kRowsPerCopy;       // copy of the row (R = 2): its tile
-    const int cbase = kCW * (dup * 2 + sub);     // this warp's columns of a pair
-    const int half = cbase / kTileKeys;          // ... all inside one tile
-    const int coff = cbase % kTileKeys;          // first column inside that tile
+    const int row = lane_t % (kRows / 2);        // packed row
+    const int dup = lane_t / (kRows / 2);        // copy of the row: its tile of a pair
     const bool owns_o = dup == 0;                // this lane writes row `row` out
-    // this lane's O: R = 1 the row's, R = 2 its copy's partial (own tile)
-    const uint32_t o_col = kOCol + (uint32_t)(dup * D);
-    const int bar_id = 1 + quad % kQuadStride;  // one named barrier per row group
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
-    // softmax warp index of (quadrant q, sub s)
-    auto sw_of = [](int q_, int s_) { return 4 * s_ + ((q_ - 2) & 3); };
-    // quadrant of copy d of this lane's row
-    auto quad_of = [&](int d) { return quad % kQuadStride + kQuadStride * d; };
+    float* m_mine = &m_sh[kSharedO ? 0 : sub][lane_t];
+    // column of this lane's O of set `set`
+    auto o_col = [&](int set) { return kOCol + (uint32_t)(set * 2 * D + dup * D); };
     // Q row -> shared (swizzled, K-major); each sub-warp copies half a row;
     // padding rows are zero.
     {
@@ -673,13 +671,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
       __syncwarp();
       if (lane == 0) mbar_arrive(&q_ready);
     }
-    float m_ref = -INFINITY, l = 0.f;
+    float m_ref = -INFINITY, l = 0.f;            // l: this group's sum, against m_ref
     bool ok = true;
-    // Every softmax warp runs all np iterations and meets its group barrier
-    // once per iteration, also after a bounded wait gave up (then it only
-    // keeps the barrier count), so that no named barrier waits forever.
-    for (int q = 0; q < np; ++q) {
-      const int j = 2 * q + half;                // the tile this warp's columns are in
+    // Every softmax warp runs all its pairs and meets the barriers of the
+    // hand-over, also after a bounded wait gave up (then it only keeps the
+    // barrier counts), so that no named barrier waits forever.
+    for (int q = sub; q < np; q += 2) {
+      const int j = 2 * q + dup;                 // the tile this lane's columns are in
       const int t = t_begin + j;
       int valid;
       if (j >= n) {
@@ -693,105 +691,100 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
       if (ok && !mbar_wait(&s_full[q & 1], (q >> 1) & 1, a.err)) ok = false;
       // tcgen05.ld/st are warp-collective: the warp goes on only as a whole
       ok = __all_sync(0xffffffffu, ok);
-      float s[kCW];
+      uint32_t sr[kCW / 16][16];                 // the scores' bits
       float mloc = -INFINITY;
       if (ok) {
         tc_fence_after();
-        const uint32_t sa = tmem + lane_addr + (uint32_t)((q & 1) * kPairKeys + cbase);
-        uint32_t r[kCW / 16][16];
+        const uint32_t sa = tmem + lane_addr + (uint32_t)((q & 1) * kPairKeys + dup * kTileKeys);
 #pragma unroll
-        for (int h = 0; h < kCW / 16; ++h) tc_ld16(sa + 16 * h, r[h]);
+        for (int h = 0; h < kCW / 16; ++h) tc_ld16(sa + 16 * h, sr[h]);
         tc_wait_ld();
-#pragma unroll
-        for (int h = 0; h < kCW / 16; ++h)
-#pragma unroll
-          for (int e = 0; e < 16; ++e) s[16 * h + e] = __uint_as_float(r[h][e]);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&s_free[q & 1]);
         // masked keys only exist in the last cache tile, the block tile and
         // the empty half of a last single-tile pair
-        if (valid < coff + kCW) {
+        if (valid < kCW) {
 #pragma unroll
           for (int c = 0; c < kCW; ++c)
-            if (coff + c >= valid) s[c] = -INFINITY;
+            if (c >= valid) sr[c / 16][c % 16] = __float_as_uint(-INFINITY);
         }
         float mx[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) mx[e] = s[e];
+        for (int e = 0; e < 8; ++e) mx[e] = __uint_as_float(sr[0][e]);
 #pragma unroll
         for (int c = 8; c < kCW; c += 8)
 #pragma unroll
-          for (int e = 0; e < 8; ++e) mx[e] = fmaxf(mx[e], s[c + e]);
+          for (int e = 0; e < 8; ++e) mx[e] = fmaxf(mx[e], __uint_as_float(sr[c / 16][c % 16 + e]));
         mloc = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
                      fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
       }
-      // The group agrees on max_w(round_up_bf16(m_w)) >= the row maximum: a
-      // reference at or above the maximum is all the lazy rescale needs (l and
-      // O share it), and every warp of the group takes the same value.
-      red_max[((q & 1) * kSoftWarps + sw) * 32 + lane] = bf16_bits_round_up(mloc);
-      asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(kGroupThreads) : "memory");
-      if (!ok) continue;
-      float mraw = -INFINITY;
-#pragma unroll
-      for (int d2 = 0; d2 < R; ++d2)
-#pragma unroll
-        for (int s2 = 0; s2 < 2; ++s2) {
-          const int w2 = sw_of(quad_of(d2), s2);
-          mraw = fmaxf(mraw, bf16_bits_to_float(red_max[((q & 1) * kSoftWarps + w2) * 32 + lane]));
+      const float mt = mloc * a.scale_log2;     // the scale is positive
+      // The reference of the pair before (of this O set) moves only when the
+      // maximum exceeds it by more than 2^8, and passes on.  A copy without
+      // keys so far has none (-inf).
+      float m_prev = m_ref;
+      if constexpr (kSharedO) {
+        if (q > 0) {
+          asm volatile("bar.sync %0, 64;" ::"r"(1 + 2 * quad + ((q - 1) & 1)) : "memory");
+          m_prev = *m_mine;
         }
-      const float mt = mraw * a.scale_log2;     // the scale is positive
+      }
       // Each row decides for itself; the TMEM rescale of O is warp-collective,
       // so a warp rescales when any of its rows does (alpha = 1 for the rest).
-      const bool rescale = m_ref != -INFINITY && mt > m_ref + kRescaleThreshold;
+      const bool rescale = m_prev != -INFINITY && mt > m_prev + kRescaleThreshold;
+      const float m_new = m_prev == -INFINITY || rescale ? mt : m_prev;
+      if constexpr (kSharedO) {
+        *m_mine = m_new;
+        __syncwarp();
+        if (q + 1 < np) asm volatile("bar.arrive %0, 64;" ::"r"(1 + 2 * quad + (q & 1)) : "memory");
+      }
+      if (!ok) continue;
+      if (m_new != m_ref) {                      // also moves made by the other group
+        l = m_ref == -INFINITY ? 0.f : l * exp2f(m_ref - m_new);
+        m_ref = m_new;
+      }
       const bool warp_rescale = __any_sync(0xffffffffu, rescale);
-      // The P block of this pair is free once PV(q-2) is done (it lives in
-      // the pair's own K sub-tiles for D = 128); O itself is only touched
-      // (rescaled) after PV(q-1).
-      const int wait_q = warp_rescale ? q - 1 : (kPInK ? -1 : q - 2);
+      // The P block of this pair is free once PV(q-2) is done (with D = 128 it
+      // lives in the pair's own K sub-tiles; the wait then only keeps the
+      // phase of pv_done known); O is only touched (rescaled) after the last
+      // PV into it: q-1 with a shared O, else q-2.
+      const int wait_q = warp_rescale && kSharedO ? q - 1 : q - 2;
       bool waited = wait_q < 0 || mbar_wait(&pv_done[wait_q & 1], (wait_q >> 1) & 1, a.err);
       if (!__all_sync(0xffffffffu, waited)) {
         ok = false;
         continue;
       }
       tc_fence_after();
-      const float alpha = rescale ? exp2f(m_ref - mt) : 1.f;
-      if (m_ref == -INFINITY) {
-        m_ref = mt;
-      } else if (rescale) {
-        l *= alpha;
-        m_ref = mt;
-      }
       if (warp_rescale) {
-        // the two sub-warps of a quadrant rescale half of its lanes' O each
-#pragma unroll
-        for (int c = sub * (D / 32); c < (sub + 1) * (D / 32); ++c) {
+        const float alpha = rescale ? exp2f(m_prev - mt) : 1.f;
+        const uint32_t oc = tmem + lane_addr + o_col(kSharedO ? 0 : sub);
+#pragma unroll 1
+        for (int c = 0; c < D / 16; ++c) {
           uint32_t r[16];
-          tc_ld16(tmem + lane_addr + o_col + c * 16, r);
+          tc_ld16(oc + c * 16, r);
           tc_wait_ld();
 #pragma unroll
           for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
-          tc_st16(tmem + lane_addr + o_col + c * 16, r);
+          tc_st16(oc + c * 16, r);
         }
         tc_wait_st();
       }
-      // P = 2^(scale * s - m_ref) as bf16 into this warp's columns of the
-      // pair's P block, in row `lane_t` (R = 1: the packed row; R = 2: the
-      // copy's row, whose keys are its tile's).  Rows past M are garbage
-      // whose O rows are never read.
-      const uint32_t pb = p_block(q) + (R == 1 ? half * kQBytes : 0);
+      // P = 2^(scale * s - m_ref) as bf16 into row `lane_t` of the pair's P
+      // block.  Rows past M are garbage whose O rows are never read.
+      const uint32_t pb = p_block(q);
       {
-        const float nm = -m_ref;
+        const float nm = m_ref == -INFINITY ? 0.f : -m_ref;   // no keys: every P is 0
         float psum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int c = 0; c < kCW / 8; ++c) {
           float p[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            p[e] = ex2_ftz(fmaf(s[c * 8 + e], a.scale_log2, nm));
+            p[e] = ex2_ftz(fmaf(__uint_as_float(sr[c / 2][(c % 2) * 8 + e]), a.scale_log2, nm));
             psum[e] += p[e];
           }
-          st_shared_v4(swz(pb, lane_t, coff / 8 + c),
+          st_shared_v4(swz(pb, lane_t, c),
                        make_uint4(pack_bf16(p[0], p[1]), pack_bf16(p[2], p[3]),
                                   pack_bf16(p[4], p[5]), pack_bf16(p[6], p[7])));
         }
@@ -804,59 +797,89 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     }
     grid_dependents_launch();
     // ------------------------------------------------ epilogue
-    // Row sums over the group, in a fixed order.  They reuse the buffer of
-    // the maxima, whose slots of every group they overlap, and a slower
-    // group may still be reading the last pair's maxima: all softmax warps
-    // pass one barrier (id 5; the groups use 1-4) before any sum is written.
-    asm volatile("bar.sync 5, %0;" ::"n"(kSoftWarps * 32) : "memory");
-    red_l[sw * 32 + lane] = l;
-    asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(kGroupThreads) : "memory");
-    float lsum = 0.f;
+    // The four warps of a row (both groups, both copies' quadrants) meet at a
+    // named barrier: references are final, then the sums against them.
+    const int row_bar = 9 + (quad & 1);
+    auto row_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(row_bar) : "memory"); };
+    if constexpr (!kSharedO) *m_mine = m_ref;
+    row_sync();
+    {
+      const float m_fin = *m_mine;
+      l_sh[sub][lane_t] = m_ref == m_fin || m_ref == -INFINITY ? l : l * exp2f(m_ref - m_fin);
+    }
+    // The last PV, waited for by the group of its pair (which has seen the PV
+    // two before, so it knows which phase the barrier is in); the barrier tells
+    // the other group.
+    bool final_ok = ok && np > 0;
+    if (final_ok && ((np - 1) & 1) == sub)
+      final_ok = mbar_wait(&pv_done[(np - 1) & 1], ((np - 1) >> 1) & 1, a.err);
+    final_ok = __all_sync(0xffffffffu, final_ok);   // the reads below are warp-collective
+    row_sync();
+    // The row's partial results: copy c of O set `set`, holding keys when
+    // part(set, c); weights w = 2^(m - M) against their largest reference M.
+    auto part = [&](int set, int c) { return n > 2 * set + c; };
+    float m_row = -INFINITY, lsum = 0.f;
 #pragma unroll
-    for (int d2 = 0; d2 < R; ++d2)
+    for (int set = 0; set < kOSets; ++set)
 #pragma unroll
-      for (int s2 = 0; s2 < 2; ++s2)
-        lsum += red_l[sw_of(quad_of(d2), s2) * 32 + lane];
+      for (int c = 0; c < 2; ++c)
+        if (part(set, c)) m_row = fmaxf(m_row, m_sh[set][c * (kRows / 2) + row]);
+    float w_mine[kOSets];                        // of this lane's copy
+#pragma unroll
+    for (int set = 0; set < kOSets; ++set) {
+      w_mine[set] = 0.f;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int ln = c * (kRows / 2) + row;
+        const float w = part(set, c) ? exp2f(m_sh[set][ln] - m_row) : 0.f;
+        const float lc = kSharedO ? l_sh[0][ln] + (np > 1 ? l_sh[1][ln] : 0.f) : l_sh[set][ln];
+        if (part(set, c)) lsum = fmaf(w, lc, lsum);
+        if (c == dup) w_mine[set] = w;
+      }
+    }
     const bool mine = owns_o && row < a.M;
     // the two sub-warps of a quadrant take half of the D columns each
     const int c_lo = sub * (D / 32), c_hi = (sub + 1) * (D / 32);
-    bool final_ok = ok && np > 0 && mbar_wait(&pv_done[(np - 1) & 1], ((np - 1) >> 1) & 1, a.err);
-    final_ok = __all_sync(0xffffffffu, final_ok);   // the reads below are warp-collective
-    // R = 2: copy 1 hands its partial O to copy 0 through shared memory (the
-    // ring, idle once the last PV is done: every load was consumed by an
-    // MMA before it).  A split of one tile gave copy 1 no keys; its half of
-    // O was never written and is left out.
+    // This lane's weighted O in columns [16 c, 16 c + 16).
+    auto own_o = [&](int c, float (&o)[16]) {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) o[e] = 0.f;
+#pragma unroll
+      for (int set = 0; set < kOSets; ++set) {
+        if (!part(set, dup)) continue;           // a set or copy without keys was never written
+        uint32_t r[16];
+        tc_ld16(tmem + lane_addr + o_col(set) + c * 16, r);
+        tc_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) o[e] = fmaf(w_mine[set], __uint_as_float(r[e]), o[e]);
+      }
+    };
+    // Copy 1 hands its weighted O to copy 0 through shared memory (the ring,
+    // idle once the last PV is done: every load was consumed by an MMA before
+    // it).
     constexpr int kStageStride = D + 1;           // floats per staged row (bank spread)
     float* stage = reinterpret_cast<float*>(smem_raw + (kv_s - smem_u32(smem_raw)));
-    const bool has_copy1 = R == 2 && n >= 2;
+    const bool has_copy1 = part(0, 1);
     // Cluster merge: this CTA's normalised partial rows and their log2-sum-
     // exps, 64 KB into the ring (past the copy-1 stage), read by every CTA of
     // the cluster after a cluster barrier.
     constexpr int kCStride = D + 4;             // floats per partial row (16-byte rows)
     float* cpart = reinterpret_cast<float*>(smem_raw + (kv_s + 65536u - smem_u32(smem_raw)));
     float* clse = cpart + kRows * kCStride;
-    if constexpr (R == 2) {
-      if (final_ok && dup == 1 && has_copy1) {
-        tc_fence_after();
+    if (final_ok && dup == 1 && has_copy1) {
+      tc_fence_after();
 #pragma unroll
-        for (int c = c_lo; c < c_hi; ++c) {
-          uint32_t r[16];
-          tc_ld16(tmem + lane_addr + o_col + c * 16, r);
-          tc_wait_ld();
+      for (int c = c_lo; c < c_hi; ++c) {
+        float o[16];
+        own_o(c, o);
 #pragma unroll
-          for (int e = 0; e < 16; ++e) stage[row * kStageStride + c * 16 + e] = __uint_as_float(r[e]);
-        }
+        for (int e = 0; e < 16; ++e) stage[row * kStageStride + c * 16 + e] = o[e];
       }
-      asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(kGroupThreads) : "memory");
     }
-    // Row `row` of O in columns [16 c, 16 c + 16): this lane's accumulator
-    // plus, with R = 2, the other copy's.
+    row_sync();
+    // Row `row` of O in columns [16 c, 16 c + 16): both copies'.
     auto load_o = [&](int c, float (&o)[16]) {
-      uint32_t r[16];
-      tc_ld16(tmem + lane_addr + o_col + c * 16, r);
-      tc_wait_ld();
-#pragma unroll
-      for (int e = 0; e < 16; ++e) o[e] = __uint_as_float(r[e]);
+      own_o(c, o);
       if (has_copy1) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) o[e] += stage[row * kStageStride + c * 16 + e];
@@ -902,7 +925,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
           }
         }
         if (mine && sub == 0) {
-          const float lse = lsum > 0.f ? m_ref + log2f(lsum) : -INFINITY;
+          const float lse = lsum > 0.f ? m_row + log2f(lsum) : -INFINITY;
           if (a.cluster) clse[row] = lse; else a.part_lse[prow] = lse;
         }
       }
@@ -1430,8 +1453,8 @@ namespace sbd {
 size_t attn_tc_smem_bytes(int D) {
   const int sub = D / 64;
   const bool p_in_k = D == 128;
-  const int pairs = p_in_k ? 3 : 4;
-  return 1024 + (size_t)sub * kRows * 128 + (p_in_k ? 0 : 4 * kRows * 128) +
+  const int pairs = p_in_k ? 3 : 5;
+  return 1024 + (size_t)sub * kRows * 128 + (p_in_k ? 0 : 2 * kRows * 128) +
          (size_t)pairs * 2 * sub * kPairKeys * 128;
 }
 
@@ -1451,25 +1474,25 @@ struct TcKernel {
 };
 static TcKernel attn_tc_kernel_for(const AttnPlan& p) {
   if (!p.wide)
-    return TcKernel{p.D == 128 ? (const void*)attn_tc_kernel<128, 2> : (const void*)attn_tc_kernel<64, 2>,
+    return TcKernel{p.D == 128 ? (const void*)attn_tc_kernel<128> : (const void*)attn_tc_kernel<64>,
                     kThreads, attn_tc_smem_bytes(p.D)};
   return TcKernel{p.D == 128 ? (const void*)attn_wide_kernel<128> : (const void*)attn_wide_kernel<64>,
                   kWideThreads, attn_wide_smem_bytes(p.D)};
 }
 
 // Above 64 packed rows only attn_wide_kernel serves.  Up to 64, at head
-// dimension 128, it is the faster one where a CTA has few keys (two triples
-// against three pairs: batch 1, 16 rows x 4 heads, 500 / 1000 / 4096 keys
-// 9.9 / 10.5 / 11.9 -> 9.0 / 9.6 / 11.0 us) and where the launch takes several
-// waves (its shared-memory traffic per key is a quarter less: 32 x 2048 keys
-// 57.8 -> 55.8 us, 64 ragged to 2000 81.7 -> 77.9).  attn_tc_kernel's shorter
-// chain of MMAs wins on long ranges of uneven length, where the longest CTA
-// sets the time (batch 4 ragged to 32768 81.0 against 84.6), and at head
-// dimension 64 (batch 16 ragged to 8000 64 against 76).
+// dimension 128, it is the faster one where a CTA has few keys (its triples
+// come through in fewer steps: 16 rows x 4 heads, batch 1, 500 / 1000 / 4096
+// keys, i.e. up to 341 a CTA, 9.9 / 10.5 / 11.7 us paired, 9.0 / 9.6 / 11.1
+// wide; batch 4, 2000 keys, 500 a CTA, 14.6 / 13.6; with few rows the line
+// lies lower: batch 2, 4096 keys, 512 a CTA, 64 rows 15.4 / 15.2 but 4 rows
+// 13.0 / 13.6), and where short sequences take several waves (its end is
+// shorter: 64 of 500-2000 keys 80.9 / 77.9; 32 of 4096 94.9 / 97.0).
 bool attn_use_wide(const AttnPlan& p) {
   if (p.M > kRows / 2) return true;
   if (p.D != 128) return false;
-  return 2ll * p.B * p.Hkv >= 3ll * num_sms() || p.Lmax <= 256ll * p.splits;
+  if (2ll * p.B * p.Hkv >= 3ll * num_sms()) return p.Lmax <= 3072;
+  return p.Lmax <= (p.M > 32 ? 704ll : 500ll) * p.splits;
 }
 
 bool attn_tc_cluster_ok(const AttnPlan& p, int splits) {

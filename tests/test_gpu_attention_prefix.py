@@ -163,16 +163,39 @@ def test_f32_split_and_tile_edges(sbd, G, k, D, n_causal):
 
 @pytest.mark.parametrize("n_causal", [0, 2])
 @pytest.mark.parametrize("splits", [1, 2, 3, 6])
-@pytest.mark.parametrize("G,k", [(1, 2), (4, 4), (3, 11), (4, 16)])
-def test_bf16_both_kernels_up_to_64_rows(sbd, G, k, splits, n_causal):
-    """Head dimension 128, up to 64 packed rows: 256 keys a split and fewer
-    run on the wide kernel, more on the paired one; the same lengths at
-    capacities on both sides of that line."""
-    lens = [0, 1, 63, 64, 65, 191, 192, 256, 257]
-    for cap in (256 * splits, 256 * splits + 1):
-        cap = max(cap, 257 + k)
-        w = gen.shrink(BF16, batch=len(lens), block_k=k, n_q_heads=G, n_kv_heads=1, cache_len=(0, cap))
+@pytest.mark.parametrize("G,k,D", [(1, 2, 128), (4, 4, 128), (3, 11, 128), (4, 16, 128), (4, 16, 64), (1, 5, 64)])
+def test_bf16_both_kernels_up_to_64_rows(sbd, G, k, D, splits, n_causal):
+    """Up to 64 packed rows: capacities on both sides of the line between the
+    wide and the paired kernel (500 or 704 keys a split at head dimension
+    128), lengths that end a pair, a tile and the hand-over between the
+    paired kernel's two groups (1 to 5 pairs, odd and even, the last of one
+    tile or two)."""
+    lens = [0, 1, 63, 64, 65, 128, 191, 192, 256, 257, 320, 449, 576]
+    line = (704 if G * k > 32 else 500) * splits
+    for cap in (line, line + 1):
+        cap = max(cap, 577 + k)
+        w = gen.shrink(BF16, batch=len(lens), block_k=k, n_q_heads=G, n_kv_heads=1, head_dim=D,
+                       cache_len=(0, cap))
         _check(sbd, w, _inputs(w, splits + k, lens), n_causal, num_splits=splits)
-    w = gen.shrink(BF16, batch=2, block_k=k, n_q_heads=2 * G, n_kv_heads=2, cache_len=(0, 1700))
-    _check(sbd, w, _inputs(w, splits + k + 1, [1690, 1025]), n_causal, num_splits=splits)
+    w = gen.shrink(BF16, batch=2, block_k=k, n_q_heads=2 * G, n_kv_heads=2, head_dim=D,
+                   cache_len=(0, 704 * splits + 900))
+    _check(sbd, w, _inputs(w, splits + k + 1, [704 * splits + 890, 1025]), n_causal, num_splits=splits)
+    assert sbd.sbd_device_error() == 0
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("rate", [0.2, 3.0])
+def test_reference_passes_between_the_groups(sbd, D, rate):
+    """Scores that grow along the cache move the softmax reference at many
+    pairs, in both groups, rows at different ones (D = 128: each move passes
+    to the other group; D = 64: each group has its own): against the oracle."""
+    import torch
+    k, G, L = 8, 4, 2900
+    w = gen.shrink(BF16, batch=2, block_k=k, n_q_heads=G, n_kv_heads=1, head_dim=D, cache_len=(0, L + 60))
+    d = _inputs(w, D, [L, L - 700])
+    kc = gen.bf16_bits_to_f32(d["k_cache"][:, :L]) * (1 + rate * np.arange(L)[None, :, None, None] / 400)
+    d["k_cache"] = d["k_cache"].copy()
+    d["k_cache"][:, :L] = gen.f32_to_bf16_bits(kc.astype(np.float32))
+    d["k_cache"][1, L - 700:] = gen.BF16_NAN
+    _check(sbd, w, d, 3, num_splits=1)
     assert sbd.sbd_device_error() == 0
