@@ -1074,8 +1074,13 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_k,
   const int n = t_end - t_begin;                  // 64-key tiles of this split
   const int nt = (n + kTriTiles - 1) / kTriTiles; // triples (the last may be short)
 
+  // The K producer only arrives: its copies need no tensor memory, and K, which
+  // the first scores wait for, goes ahead of V (first iteration, batch 8,
+  // ragged to 4001 keys 32.6 -> 30.4 us; batch 16, 8192 keys 90.3 -> 88.1; with
+  // V's producer early as well 31.5 and 90.0).
   tc_fence_before();
-  __syncthreads();
+  if (warp == 0) asm volatile("bar.arrive 15, %0;" ::"n"(kWideThreads) : "memory");
+  else asm volatile("bar.sync 15, %0;" ::"n"(kWideThreads) : "memory");
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
 
