@@ -3,8 +3,8 @@
 // Eqs. 6-7 and Algorithm 3 "compute probabilities"; EB input of Eq. 3).
 //
 // Kernels, in launch order on one stream:
-//   compact_rows_kernel  gathers the hidden rows of masked positions into a
-//                        dense [rows_alloc, H] buffer and a row map; writes
+//   compact_rows_kernel  (bf16) gathers the hidden rows of masked positions into
+//                        a dense [rows_alloc, H] buffer and a row map; writes
 //                        entropy = +inf / token = -1 for unmasked positions;
 //   head_pair_kernel     (bf16) the LM head on CTA pairs (clusters of 2) with
 //                        2-SM tcgen05 MMAs of M = 256: W and the masked
@@ -23,7 +23,8 @@
 //                        quadrant, alternate 16-column chunks) reduce each
 //                        logit column over the lanes.  The fallback where no
 //                        cluster of two fits or the vocabulary is one tile;
-//   head_f32_kernel      (fp32) the same reduction over exact fp32 FMAs;
+//   head_f32_kernel      (fp32) the same over fp32 FMAs, finding the masked rows
+//                        itself;
 //   head_combine_kernel  merges the per-CTA statistics of each row into the
 //                        entropy (nats), the token and, when asked for, the
 //                        confidence max_v p_v = 1 / S.
@@ -1528,6 +1529,7 @@ constexpr int kF32HeadThreads = 32 * kF32HeadWarps;
 constexpr int kF32Cols = 32;
 constexpr int kF32Stages = 4;
 constexpr int kF32Rows = 32;                         // rows of a group
+constexpr int kF32MaxRows = 512;                     // B k at most
 constexpr int kF32StageFloats = (kBM + kF32Rows) * kF32Cols;
 constexpr size_t kF32SmemBytes = sizeof(float) * kF32Stages * kF32StageFloats;
 static_assert(kF32HeadWarps * 16 * kBM <= kF32Stages * kF32StageFloats, "the partial logits fit the ring");
@@ -1540,8 +1542,9 @@ __device__ __forceinline__ int f32_w_at(int row, int c) {
 
 struct F32HeadTile {
   const float* w;          // W row v0
-  const float* hidden;     // hidden row r0
-  int H, v_left, rows;     // columns; vocabulary rows from v0; rows to load (past R: zeros)
+  const float* hidden;     // hidden [B k, H]
+  const int* map;          // the group's hidden rows
+  int H, v_left, rows;     // columns; vocabulary rows from v0; rows of the group
 };
 
 // Partial logits of the tile into ring as [warp][2 TR rows][kBM], up to 16
@@ -1554,6 +1557,7 @@ __device__ __forceinline__ void f32_tile_ring(const F32HeadTile& t, float* ring)
   const int c_ld = tid & 7, r_ld = tid >> 3;         // staged 16-byte column, first row
   const int vl = lane & 15;                          // ids vl + 16 j
   const int row0 = (lane >> 4) * TR;                 // rows row0 + r
+  const float* h_row = t.hidden + (size_t)(r_ld < t.rows ? t.map[r_ld] : 0) * t.H;
   auto load = [&](int chunk) {
     float* ws = ring + (chunk % kF32Stages) * kF32StageFloats;
     float* hs = ws + kBM * kF32Cols;
@@ -1566,8 +1570,9 @@ __device__ __forceinline__ void f32_tile_ring(const F32HeadTile& t, float* ring)
       const bool ok = in && row < t.v_left;
       cp_async16(ws + f32_w_at(row, c_ld), ok ? wp + (size_t)row * t.H : t.w, ok);
     }
-    if (r_ld < t.rows)
-      cp_async16(hs + r_ld * kF32Cols + 4 * c_ld, t.hidden + (size_t)r_ld * t.H + (in ? col : 0), in);
+    // (rows past the group's last are zeros, up to a multiple of 8)
+    if (r_ld < ((t.rows + 7) & ~7))
+      cp_async16(hs + r_ld * kF32Cols + 4 * c_ld, h_row + (in ? col : 0), in && r_ld < t.rows);
   };
 #pragma unroll
   for (int c = 0; c < kF32Stages - 1; ++c) {
@@ -1626,6 +1631,7 @@ __device__ __forceinline__ void f32_tile_cols(const F32HeadTile& t, float* ring)
   constexpr int kIter = kBM * 8 / kF32HeadThreads;
   constexpr int kBuf = kF32Cols * (kBM + kF32Rows);  // floats of a buffer
   float4 wr[kIter], hr;
+  const float* h_row = t.hidden + (size_t)(r_ld < t.rows ? t.map[r_ld] : 0) * t.H;
   auto fetch = [&](int chunk) {
     const int col = chunk * kF32Cols + 4 * c_ld;
     const bool in = col < t.H;
@@ -1636,9 +1642,8 @@ __device__ __forceinline__ void f32_tile_cols(const F32HeadTile& t, float* ring)
                   ? __ldg(reinterpret_cast<const float4*>(t.w + (size_t)row * t.H + col))
                   : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    hr = in && r_ld < t.rows
-             ? *reinterpret_cast<const float4*>(t.hidden + (size_t)r_ld * t.H + col)
-             : make_float4(0.f, 0.f, 0.f, 0.f);
+    hr = in && r_ld < t.rows ? *reinterpret_cast<const float4*>(h_row + col)
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
   };
   const int turn_st = 8 * (c_ld >> 1);               // of columns 4 c_ld .. + 3
   auto put = [&](float* buf) {
@@ -1708,14 +1713,49 @@ __device__ __forceinline__ void f32_tile_cols(const F32HeadTile& t, float* ring)
 
 template <bool kPhilox>
 __global__ void __launch_bounds__(kF32HeadThreads, 2)
-head_f32_kernel(const float* __restrict__ hidden_c, const float* __restrict__ w,
-                const float* __restrict__ gumbel, const int32_t* __restrict__ row_map,
-                const int32_t* __restrict__ n_rows, float tau, int V, int H, int rows_alloc,
-                float4* __restrict__ part_msTb, int32_t* __restrict__ part_idx,
-                uint4 philox_sk) {
+head_f32_kernel(const float* __restrict__ hidden, const float* __restrict__ w,
+                const float* __restrict__ gumbel, const uint8_t* __restrict__ masked, int BK,
+                int32_t* __restrict__ row_map, int32_t* __restrict__ n_rows, float tau, int V,
+                int H, int rows_alloc, float4* __restrict__ part_msTb,
+                int32_t* __restrict__ part_idx, float* __restrict__ entropy,
+                int32_t* __restrict__ token, float* __restrict__ confidence, uint4 philox_sk) {
   extern __shared__ __align__(16) float f32_smem[];
+  // The masked rows in order: every CTA finds them for itself (B k <= 512
+  // flags), the first one writes them out for the merge, and the unmasked
+  // rows' results; the hidden rows are read where they are.  A kernel of its own
+  // that did this and copied the rows, as for bf16, cost a launch: 1-3 rows of
+  // hidden 256, 512 ids 8.8 -> 7.6 us, 32 rows of 2048, 32003 ids 132 -> 128.5.
+  __shared__ int rows_sh[kF32MaxRows], count_sh[kF32MaxRows / 32];
   grid_dependency_wait();
-  const int R = *n_rows;
+  for (int i0 = 0; i0 < kF32MaxRows; i0 += kF32HeadThreads) {
+    const int i = i0 + threadIdx.x;
+    const unsigned bal = __ballot_sync(0xffffffffu, i < BK && masked[i] != 0);
+    if ((threadIdx.x & 31) == 0) count_sh[i / 32] = __popc(bal);
+  }
+  __syncthreads();
+  int R = 0;
+  for (int i0 = 0; i0 < kF32MaxRows; i0 += kF32HeadThreads) {
+    const int i = i0 + threadIdx.x, ln = threadIdx.x & 31;
+    // the counts of the groups of 32 before this one, and of all
+    const int c = ln < kF32MaxRows / 32 ? count_sh[ln] : 0;
+    const int before = __reduce_add_sync(0xffffffffu, ln < i / 32 ? c : 0);
+    R = __reduce_add_sync(0xffffffffu, c);
+    const bool live = i < BK && masked[i] != 0;
+    const unsigned bal = __ballot_sync(0xffffffffu, live);
+    const int at = before + __popc(bal & ((1u << ln) - 1u));
+    if (live) rows_sh[at] = i;
+    if (blockIdx.x == 0 && i < BK) {
+      if (live) {
+        row_map[at] = i;
+      } else {
+        entropy[i] = INFINITY;
+        token[i] = -1;
+        if (confidence) confidence[i] = 0.f;
+      }
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *n_rows = R;
+  __syncthreads();
   const int v0 = blockIdx.x * kBM;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool noisy = tau != 0.f && (kPhilox || gumbel != nullptr);
@@ -1725,10 +1765,11 @@ head_f32_kernel(const float* __restrict__ hidden_c, const float* __restrict__ w,
     const int nr = min(kF32Rows, R - r0);
     F32HeadTile t;
     t.w = w + (size_t)v0 * H;
-    t.hidden = hidden_c + (size_t)r0 * H;
+    t.hidden = hidden;
+    t.map = rows_sh + r0;
     t.H = H;
     t.v_left = V - v0;
-    t.rows = (nr + 7) & ~7;                          // hidden_c has zero rows past R
+    t.rows = nr;
     int zrows = 32, parts = 4;                       // [parts][zrows][kBM] partial logits
     if (nr <= 8) {
       f32_tile_ring<4>(t, f32_smem);
@@ -1751,7 +1792,7 @@ head_f32_kernel(const float* __restrict__ hidden_c, const float* __restrict__ w,
 #pragma unroll
       for (int j = 0; j < 4; ++j) g[i][j] = 0.f;
       if (noisy && row < nr) {
-        const int n = row_map[r0 + row];
+        const int n = rows_sh[r0 + row];
         if constexpr (kPhilox) {
           // philox_sk = (seed low, seed high, offset low, offset high); the
           // lane's four ids are the four words of one call
@@ -1883,7 +1924,7 @@ head_combine_kernel(const float4* __restrict__ part_msTb, const int32_t* __restr
 
 // ------------------------------------------------------------ workspace
 struct HeadWs {
-  uint8_t* hidden_c;
+  uint8_t* hidden_c;       // the masked rows (bf16 only)
   int32_t* row_map;
   int32_t* n_rows;
   float4* part_msTb;
@@ -1895,8 +1936,10 @@ HeadWs head_ws_layout(const sbd::HeadPlan& p, void* base) {
   HeadWs w;
   const uintptr_t c = reinterpret_cast<uintptr_t>(base);
   size_t off = 0;
-  const size_t elem = p.bf16 ? 2 : 4;
   w.hidden_c = reinterpret_cast<uint8_t*>(c + off);
+  // (fp32 reads its rows where they are, and keeps the size: the fixed scratch
+  // of the no-allocation call takes the same shapes as ever)
+  const size_t elem = p.bf16 ? 2 : 4;
   off = sbd::align_up(off + (size_t)p.rows_alloc * p.H * elem, 256);
   w.row_map = reinterpret_cast<int32_t*>(c + off);
   off = sbd::align_up(off + (size_t)p.rows_alloc * 4, 256);
@@ -2048,25 +2091,24 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
   const int BK = p.B * p.k;
   if (BK == 0) return SBD_OK;
   HeadWs W = head_ws_layout(p, ws);
-  const int elem = p.bf16 ? 2 : 4;
   sbd_status s;
-  {
-    const uint8_t* hid = (const uint8_t*)hidden;
-    int bk = BK, rb = p.H * elem;
-    uint8_t* hc = W.hidden_c;
-    int32_t* rm = W.row_map;
-    int32_t* nr = W.n_rows;
-    void* args[] = {(void*)&hid, (void*)&masked,  (void*)&bk,    (void*)&rb,
-                    (void*)&hc,  (void*)&rm,      (void*)&nr,    (void*)&entropy,
-                    (void*)&token, (void*)&confidence};
-    s = launch_pdl((const void*)compact_rows_kernel, dim3(p.rows_alloc), dim3(256), 0, st, args,
-                   "compact_rows_kernel launch");
-    if (s != SBD_OK) return s;
-  }
   cudaError_t e;
   int* err = device_error_word();
   int n_parts = p.n_ctas;   // CTAs that write per-row partials
   if (p.bf16) {
+    {
+      const uint8_t* hid = (const uint8_t*)hidden;
+      int bk = BK, rb = p.H * 2;
+      uint8_t* hc = W.hidden_c;
+      int32_t* rm = W.row_map;
+      int32_t* nr = W.n_rows;
+      void* args[] = {(void*)&hid, (void*)&masked,  (void*)&bk,    (void*)&rb,
+                      (void*)&hc,  (void*)&rm,      (void*)&nr,    (void*)&entropy,
+                      (void*)&token, (void*)&confidence};
+      s = launch_pdl((const void*)compact_rows_kernel, dim3(p.rows_alloc), dim3(256), 0, st, args,
+                     "compact_rows_kernel launch");
+    }
+    if (s != SBD_OK) return s;
     CUtensorMap tw, th, th64, th128;
     {
       const uint64_t dims[2] = {(uint64_t)p.H, (uint64_t)p.V};
@@ -2163,10 +2205,11 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
                    n_pairs > 0 ? 2 : 1);
     if (s != SBD_OK) return s;
   } else {
-    const float* hc = (const float*)W.hidden_c;
+    const float* hf = (const float*)hidden;
     const float* wf = (const float*)w;
-    const int32_t* rm = W.row_map;
-    const int32_t* nr = W.n_rows;
+    int bk = BK;
+    int32_t* rm = W.row_map;
+    int32_t* nr = W.n_rows;
     int V = p.V, H = p.H, ra = p.rows_alloc;
     float4* pm = W.part_msTb;
     int32_t* pi = W.part_idx;
@@ -2174,9 +2217,10 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     if (philox)
       sk = make_uint4((uint32_t)philox->seed, (uint32_t)(philox->seed >> 32),
                       (uint32_t)philox->offset, (uint32_t)(philox->offset >> 32));
-    void* args[] = {(void*)&hc, (void*)&wf, (void*)&gumbel, (void*)&rm, (void*)&nr,
-                    (void*)&tau, (void*)&V,  (void*)&H,      (void*)&ra, (void*)&pm,
-                    (void*)&pi, (void*)&sk};
+    void* args[] = {(void*)&hf, (void*)&wf, (void*)&gumbel,  (void*)&masked, (void*)&bk,
+                    (void*)&rm, (void*)&nr, (void*)&tau,     (void*)&V,      (void*)&H,
+                    (void*)&ra, (void*)&pm, (void*)&pi,      (void*)&entropy, (void*)&token,
+                    (void*)&confidence, (void*)&sk};
     const void* fn =
         philox ? (const void*)head_f32_kernel<true> : (const void*)head_f32_kernel<false>;
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32SmemBytes);

@@ -105,6 +105,24 @@ def test_f32_row_groups(sbd, R, V, H, philox):
     assert sbd.sbd_device_error() == 0
 
 
+@pytest.mark.parametrize("which", ["none", "all", "first", "last", "odd", "run"])
+@pytest.mark.parametrize("B,k", [(1, 1), (1, 31), (4, 8), (3, 11), (15, 17), (8, 32), (257, 1), (16, 32)])
+def test_f32_finds_the_masked_rows(sbd, B, k, which):
+    """The fp32 kernel's own list of masked rows: counts around its words of 32
+    flags and its 256 threads, up to 512; nothing, everything, one row at either
+    end, every other row and a run that crosses the words' edges masked."""
+    N = B * k
+    m = np.zeros(N, dtype=np.uint8)
+    m[{"none": slice(0, 0), "all": slice(0, N), "first": slice(0, 1), "last": slice(N - 1, N),
+       "odd": slice(1, N, 2), "run": slice(N // 3, 2 * N // 3 + 1)}[which]] = 1
+    w = gen.shrink(gen.get_workload("tiny_f32"), batch=B, block_k=k, vocab=37, hidden=12)
+    d = dict(step_inputs(w, seed=N))
+    d["masked"] = m.reshape(B, k)
+    ent, tok = run_head(sbd, d, "f32", 1.0)
+    assert compare_head(d, "f32", 1.0, ent, tok) <= 1
+    assert sbd.sbd_device_error() == 0
+
+
 @pytest.mark.parametrize("B,k,V,H", [(1, 1, 1000, 256), (1, 16, 4096 + 5, 512), (2, 16, 3000, 128),
                                      (3, 7, 777, 64), (16, 16, 2100, 256), (1, 17, 500, 128),
                                      (10, 30, 999, 64), (16, 32, 1500, 128),
