@@ -3,7 +3,8 @@
 // Eqs. 6-7 and Algorithm 3 "compute probabilities"; EB input of Eq. 3).
 //
 // Kernels, in launch order on one stream:
-//   compact_rows_kernel  (bf16) gathers the hidden rows of masked positions into
+//   compact_rows_kernel  (bf16 above 32 rows, or without CTA pairs) gathers the
+//                        hidden rows of masked positions into
 //                        a dense [rows_alloc, H] buffer and a row map; writes
 //                        entropy = +inf / token = -1 for unmasked positions;
 //   head_pair_kernel     (bf16) the LM head on CTA pairs (clusters of 2) with
@@ -419,6 +420,15 @@ struct HeadArgs {
   uint32_t seed_lo, seed_hi, off_lo, off_hi;   // counter-based noise (kPhilox)
   const int32_t* row_map;
   const int32_t* n_rows;
+  // pair kernel, rows in place: the flags of all n_flags <= kInPlaceRows rows
+  // (NULL: the compaction kernel ran), and what that kernel writes otherwise
+  const uint8_t* masked;
+  int n_flags;
+  int32_t* row_map_out;
+  int32_t* n_rows_out;
+  float* entropy;
+  int32_t* token;
+  float* confidence;
   float4* part_msTb;     // [gridDim.x][rows_alloc]
   int32_t* part_idx;
   int* err;
@@ -990,9 +1000,19 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
         tma_prefetch_l2_2d(&tmap_w, kb * kBK, (2 * (tk / a.ksplit) + rank) * w_rows);
     }
   }
-  // Everything below reads what the compaction kernel wrote.
+  // Everything below reads what the kernels before it wrote.
   grid_dependency_wait();
-  const int R = kLinear ? a.linear_rows : *a.n_rows;
+  // Up to kInPlaceRows rows nothing is compacted: all of them go through the
+  // MMAs, which take that many columns in any case, unless none is masked.
+  const bool in_place = !kLinear && a.masked != nullptr;
+  uint32_t flags = 0;
+  int R;
+  if (in_place) {
+    flags = __ballot_sync(0xffffffffu, lane < a.n_flags && a.masked[lane] != 0);
+    R = flags != 0 ? a.n_flags : 0;
+  } else {
+    R = kLinear ? a.linear_rows : *a.n_rows;
+  }
   // The layout: hidden rows on the lanes above kPairVocabLanesMax live rows,
   // vocabulary rows on the lanes up to it.
   const bool rows_mode = kLinear || R > kPairVocabLanesMax;
@@ -1082,9 +1102,23 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
   }
   if (!rows_mode && warp >= 2) {
     for (int i = threadIdx.x - 64; i < n_eff; i += kEpiThreads) {
-      rmap[i] = i < R ? a.row_map[i] : 0;
+      // (in place, a row that is not masked reads the first masked row's noise,
+      // which costs no traffic; its statistics are not used)
+      rmap[i] = i >= R ? 0 : !in_place ? a.row_map[i] : (flags >> i) & 1u ? i : __ffs(flags) - 1;
       for (int w = 0; w < 4; ++w) store_stats(wstats(w), i, rowstats_empty());
     }
+  }
+  if (in_place && blockIdx.x == 0 && warp == 1) {
+    if (lane < a.n_flags) {
+      const bool is_live = (flags >> lane) & 1u;
+      a.row_map_out[lane] = is_live ? lane : -1;
+      if (!is_live) {
+        a.entropy[lane] = INFINITY;
+        a.token[lane] = -1;
+        if (a.confidence) a.confidence[lane] = 0.f;
+      }
+    }
+    if (lane == 0) *a.n_rows_out = R;
   }
   // Both CTAs run and their barriers are initialised before either one
   // signals the other's; the pair then allocates its tensor memory.
@@ -1877,7 +1911,7 @@ head_combine_kernel(const float4* __restrict__ part_msTb, const int32_t* __restr
   const int lane = threadIdx.x & 31;
   if (r >= rows_alloc) return;
   const int rows = *n_rows;
-  const int row = row_map[r];        // read before the check: r < rows_alloc
+  const int row = row_map[r];        // read before the check: r < rows_alloc; -1: not masked
   RowStats s = rowstats_empty();
   for (int c0 = 0; c0 < n_parts; c0 += 32 * kPerLane) {
     float4 v[kPerLane];
@@ -1903,7 +1937,7 @@ head_combine_kernel(const float4* __restrict__ part_msTb, const int32_t* __restr
       }
     }
   }
-  if (r >= rows) return;
+  if (r >= rows || row < 0) return;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     RowStats t;
@@ -1973,6 +2007,15 @@ size_t head_smem_bytes(int rows_alloc) {
 // of two and for a vocabulary of one tile); its shared memory is the ring
 // alone.
 constexpr int kPairMinRows = 16;
+// Rows up to which the pair kernel takes the hidden rows where they are instead
+// of compacted ones: its B side is padded to 32 rows in any case, so the rows
+// that are not masked cost nothing in the MMAs, and a launch on the critical
+// path goes.  16 rows of 4096, 128256 ids: 158.7 -> 156.7 us; 4 rows of 2048,
+// 32000 ids: 30.5 -> 29.5; 32 rows, all masked, 160.8 -> 159.0, 3 of them
+// 159.4 -> 158.9 (32000 ids, in-kernel noise: 32.8 -> 33.1).  Above 32 rows the
+// padded N would grow with rows that are not masked.  (Compaction by TMA
+// gather4 loads of the masked rows: 16 rows 158.5 -> 168.8, 64 rows 168 -> 246.)
+constexpr int kInPlaceRows = 32;
 // its ring: what is left of the 227 KB of a CTA next to its static shared
 // memory (barriers and 2.5 KB of row statistics) and the 1 KB alignment
 constexpr int kPairRingBytes = 222 * 1024;
@@ -2096,7 +2139,22 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
   int* err = device_error_word();
   int n_parts = p.n_ctas;   // CTAs that write per-row partials
   if (p.bf16) {
-    {
+    // CTA pairs from kPairMinRows allocated rows: as many as the device holds
+    // at once, the pair tiles need and the workspace has partials for
+    // (p.n_ctas), an even number when there may be two row groups.
+    const void* fn_pair = philox ? (const void*)head_pair_kernel<true, false>
+                                 : (const void*)head_pair_kernel<false, false>;
+    const int pair_tiles = (p.V + 2 * kBM - 1) / (2 * kBM);
+    const int n_groups_max = p.rows_alloc > 2 * kPairRows ? 2 : 1;
+    int n_pairs = 0;
+    if (p.rows_alloc >= kPairMinRows && p.n_ctas >= 2) {
+      n_pairs = head_pair_slots(fn_pair);
+      if (n_pairs > pair_tiles * n_groups_max) n_pairs = pair_tiles * n_groups_max;
+      if (n_pairs > p.n_ctas / 2) n_pairs = p.n_ctas / 2;
+      if (n_groups_max == 2) n_pairs &= ~1;
+    }
+    const bool in_place = n_pairs > 0 && BK <= kInPlaceRows;
+    if (!in_place) {
       const uint8_t* hid = (const uint8_t*)hidden;
       int bk = BK, rb = p.H * 2;
       uint8_t* hc = W.hidden_c;
@@ -2107,8 +2165,8 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
                       (void*)&token, (void*)&confidence};
       s = launch_pdl((const void*)compact_rows_kernel, dim3(p.rows_alloc), dim3(256), 0, st, args,
                      "compact_rows_kernel launch");
+      if (s != SBD_OK) return s;
     }
-    if (s != SBD_OK) return s;
     CUtensorMap tw, th, th64, th128;
     {
       const uint64_t dims[2] = {(uint64_t)p.H, (uint64_t)p.V};
@@ -2119,23 +2177,24 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
       if (s != SBD_OK) return s;
     }
     {
-      const uint64_t dims[2] = {(uint64_t)p.H, (uint64_t)p.rows_alloc};
+      void* rows = in_place ? (void*)hidden : (void*)W.hidden_c;
+      const uint64_t dims[2] = {(uint64_t)p.H, (uint64_t)(in_place ? BK : p.rows_alloc)};
       const uint64_t strides[1] = {(uint64_t)p.H * 2};
       const uint32_t box[2] = {(uint32_t)kBK, 16u};
-      s = encode_tensor_map(&th, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)W.hidden_c, dims,
+      s = encode_tensor_map(&th, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, rows, dims,
                             strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
       if (s != SBD_OK) return s;
       th64 = th;
       th128 = th;
       if (p.rows_alloc >= 64) {
         const uint32_t box64[2] = {(uint32_t)kBK, 64u};
-        s = encode_tensor_map(&th64, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)W.hidden_c, dims,
+        s = encode_tensor_map(&th64, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, rows, dims,
                               strides, box64, CU_TENSOR_MAP_SWIZZLE_128B);
         if (s != SBD_OK) return s;
       }
       if (p.rows_alloc >= 128) {
         const uint32_t box128[2] = {(uint32_t)kBK, 128u};
-        s = encode_tensor_map(&th128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)W.hidden_c,
+        s = encode_tensor_map(&th128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, rows,
                               dims, strides, box128, CU_TENSOR_MAP_SWIZZLE_128B);
         if (s != SBD_OK) return s;
       }
@@ -2148,6 +2207,13 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     a.off_hi = philox ? (uint32_t)(philox->offset >> 32) : 0u;
     a.row_map = W.row_map;
     a.n_rows = W.n_rows;
+    a.masked = in_place ? masked : nullptr;
+    a.n_flags = BK;
+    a.row_map_out = W.row_map;
+    a.n_rows_out = W.n_rows;
+    a.entropy = entropy;
+    a.token = token;
+    a.confidence = confidence;
     a.part_msTb = W.part_msTb;
     a.part_idx = W.part_idx;
     a.err = err;
@@ -2163,20 +2229,6 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     a.part_y = nullptr;
     a.h_big = p.rows_alloc >= 128 ? 128 : (p.rows_alloc >= 64 ? 64 : 16);
     a.tau = tau;
-    // CTA pairs from kPairMinRows allocated rows: as many as the device holds
-    // at once, the pair tiles need and the workspace has partials for
-    // (p.n_ctas), an even number when there may be two row groups.
-    const void* fn_pair = philox ? (const void*)head_pair_kernel<true, false>
-                                 : (const void*)head_pair_kernel<false, false>;
-    const int pair_tiles = (p.V + 2 * kBM - 1) / (2 * kBM);
-    const int n_groups_max = p.rows_alloc > 2 * kPairRows ? 2 : 1;
-    int n_pairs = 0;
-    if (p.rows_alloc >= kPairMinRows && p.n_ctas >= 2) {
-      n_pairs = head_pair_slots(fn_pair);
-      if (n_pairs > pair_tiles * n_groups_max) n_pairs = pair_tiles * n_groups_max;
-      if (n_pairs > p.n_ctas / 2) n_pairs = p.n_ctas / 2;
-      if (n_groups_max == 2) n_pairs &= ~1;
-    }
     const void* fn;
     size_t smem;
     if (n_pairs > 0) {

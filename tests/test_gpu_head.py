@@ -197,6 +197,33 @@ def test_pair_kernel_without_masked_rows(sbd, philox):
     assert sbd.sbd_device_error() == 0
 
 
+@pytest.mark.parametrize("which", ["none", "all", "first", "last", "odd"])
+@pytest.mark.parametrize("B,k", [(1, 1), (1, 15), (2, 8), (1, 17), (31, 1), (4, 8), (3, 11)])
+def test_bf16_rows_in_place(sbd, B, k, which):
+    """Up to 32 rows the pair kernel reads every hidden row where it is: rows
+    that are not masked may hold anything (NaN here) without touching the
+    others, and none masked means no work; 33 rows are compacted.  Noise from
+    the buffer and the kernel's own, which must agree bit for bit."""
+    import torch
+    N = B * k
+    m = np.zeros(N, dtype=np.uint8)
+    m[{"none": slice(0, 0), "all": slice(0, N), "first": slice(0, 1), "last": slice(N - 1, N),
+       "odd": slice(1, N, 2)}[which]] = 1
+    w = gen.shrink(gen.get_workload("llama8b_k16"), batch=B, block_k=k, vocab=801, hidden=192,
+                   cache_len=64)
+    d = dict(step_inputs(w, seed=N))
+    d["masked"] = m.reshape(B, k)
+    ids = torch.arange(N, dtype=torch.int32, device="cuda")
+    d["gumbel"] = sbd.sbd_gumbel_philox(ids, 801, 5, 2).cpu().numpy().reshape(B, k, 801)
+    hid, W, mk = to_dev(d["hidden"], "bf16"), to_dev(d["w"], "bf16"), torch.from_numpy(d["masked"]).cuda()
+    hid[mk == 0] = float("nan")
+    ent, tok = sbd.sbd_head_entropy_sample(hid, W, mk, torch.from_numpy(d["gumbel"]).cuda(), 1.0)
+    assert compare_head(d, "bf16", 1.0, ent.cpu().numpy(), tok.cpu().numpy()) <= 1
+    e2, t2 = sbd.sbd_head_entropy_sample_philox(hid, W, mk, 5, 2, 1.0)
+    assert torch.equal(e2, ent) and torch.equal(t2, tok)
+    assert sbd.sbd_device_error() == 0
+
+
 def test_bf16_uniform_and_one_hot_rows(sbd):
     """Closed forms through the kernel: zero hidden -> uniform -> log V;
     a huge logit -> entropy 0 and that token."""
