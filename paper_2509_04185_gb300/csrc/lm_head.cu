@@ -424,6 +424,7 @@ struct HeadArgs {
   // (NULL: the compaction kernel ran), and what that kernel writes otherwise
   const uint8_t* masked;
   int n_flags;
+  int prefetch;         // pair kernel: boxes of a CTA's first W rows brought into L2 early
   int32_t* row_map_out;
   int32_t* n_rows_out;
   float* entropy;
@@ -999,6 +1000,11 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
       if (kb < a.H / kBK)
         tma_prefetch_l2_2d(&tmap_w, kb * kBK, (2 * (tk / a.ksplit) + rank) * w_rows);
     }
+  }
+  if constexpr (!kLinear) {
+    // (as above: L2 only)
+    if (warp == 0 && lane < a.prefetch)
+      tma_prefetch_l2_2d(&tmap_w, lane * kBK, (2 * pair + rank) * kBM);
   }
   // Everything below reads what the kernels before it wrote.
   grid_dependency_wait();
@@ -2016,6 +2022,16 @@ constexpr int kPairMinRows = 16;
 // padded N would grow with rows that are not masked.  (Compaction by TMA
 // gather4 loads of the masked rows: 16 rows 158.5 -> 168.8, 64 rows 168 -> 246.)
 constexpr int kInPlaceRows = 32;
+// Without the compaction kernel in between, the pair kernel comes up while the
+// kernel before it (attention, in a step) still runs, and its first boxes of W
+// are brought into L2 meanwhile; they are read from there once that kernel is
+// done.  16 boxes: 32000 ids of 2048 29.3 -> 27.7 us (8 boxes 28.4; 32 27.8),
+// 50304 of 1024 24.0 -> 23.2, 151936 of 4096 182.8 -> 180.7, 128256 158.3 ->
+// 156.1.  A W that stays in L2 from call to call only loses (82 MB: 24.8 ->
+// 25.7 us; 41 MB 17.2 -> 18.0), and W below about this size does.  (With no row
+// masked they are read for nothing: 5.6 -> 6.4 us.)
+constexpr int kPrefetchBoxes = 16;
+constexpr size_t kPrefetchMinBytes = 96u << 20;
 // its ring: what is left of the 227 KB of a CTA next to its static shared
 // memory (barriers and 2.5 KB of row statistics) and the 1 KB alignment
 constexpr int kPairRingBytes = 222 * 1024;
@@ -2209,6 +2225,9 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     a.n_rows = W.n_rows;
     a.masked = in_place ? masked : nullptr;
     a.n_flags = BK;
+    a.prefetch = 0;
+    if (in_place && (size_t)p.V * p.H * 2 >= kPrefetchMinBytes)
+      a.prefetch = p.H / kBK < kPrefetchBoxes ? p.H / kBK : kPrefetchBoxes;
     a.row_map_out = W.row_map;
     a.n_rows_out = W.n_rows;
     a.entropy = entropy;
