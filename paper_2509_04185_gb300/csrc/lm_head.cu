@@ -420,16 +420,6 @@ struct HeadArgs {
   uint32_t seed_lo, seed_hi, off_lo, off_hi;   // counter-based noise (kPhilox)
   const int32_t* row_map;
   const int32_t* n_rows;
-  // pair kernel, rows in place: the flags of all n_flags <= kInPlaceRows rows
-  // (NULL: the compaction kernel ran), and what that kernel writes otherwise
-  const uint8_t* masked;
-  int n_flags;
-  int prefetch;         // pair kernel: boxes of a CTA's first W rows brought into L2 early
-  int32_t* row_map_out;
-  int32_t* n_rows_out;
-  float* entropy;
-  int32_t* token;
-  float* confidence;
   float4* part_msTb;     // [gridDim.x][rows_alloc]
   int32_t* part_idx;
   int* err;
@@ -444,6 +434,16 @@ struct HeadArgs {
   int w_rows;           // kLinear, pairs: W rows of a unit per CTA (a multiple of 16 up to 128)
   int k_cluster;        // kLinear: the ranges of a tile form one cluster and add up there
   float* part_y;        // kLinear, ksplit > 1: fp32 partials [ksplit][linear_rows][V]
+  // kInPlace: the flags of all n_flags rows, and what the compaction kernel
+  // writes otherwise
+  const uint8_t* masked;
+  int n_flags;
+  int prefetch;         // boxes of a CTA's first W rows brought into L2 early
+  int32_t* row_map_out;
+  int32_t* n_rows_out;
+  float* entropy;
+  int32_t* token;
+  float* confidence;
 };
 
 // kPhilox: the Gumbel noise is generated in the epilogue (philox.cuh)
@@ -656,7 +656,7 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
       const int quad = warp & 3;               // TMEM lanes 32*quad .. 32*quad+31
       const StatsRef my_stats = wstats(quad);
       const int sub = (warp - 2) / 4;          // chunks sub, sub + n_sub, ... of 16 columns
-      const bool noisy = !kLinear && a.tau != 0.f && (kPhilox || a.gumbel != nullptr);
+      const bool noisy = kPhilox || (!kLinear && a.tau != 0.f && a.gumbel != nullptr);
       const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
       int local = 0;
       for (int u = blockIdx.x; sub < n_sub && u < n_units; u += gridDim.x, ++local) {
@@ -927,7 +927,7 @@ __device__ __forceinline__ void fold_scores16(RowStats& st, const float (&z)[16]
 // Per call at V = 128256, H = 4096 (bursts), two logarithms a logit against
 // this: 200 rows 227 -> 205 us, 256 rows 225 -> 210, 320 rows 435 -> 385, 512
 // rows 460 -> 380 (the noise buffer: 203, 209, 346, 351); V = 151936, 512
-// rows, under the power cap 486 -> 450.  Most of the rest are the generator's
+// rows, under the power cap 480 -> 441-453.  Most of the rest are the generator's
 // rounds.  (Round keys from the host made no difference.)
 template <bool kFull>
 __device__ __forceinline__ void fold_words16(RowStats& st, const float (&z)[16],
@@ -961,7 +961,11 @@ __device__ __forceinline__ void fold_words16(RowStats& st, const float (&z)[16],
 // always in the rows layout, the epilogue storing each row's outputs; with
 // a.ksplit > 1 each (pair tile, K range) is a unit and the epilogue stores
 // fp32 partials for linear_reduce_kernel.
-template <bool kPhilox, bool kLinear>
+// kInPlace: up to kInPlaceRows rows, read where they are (no compaction): all of
+// them go through the MMAs, which take that many columns in any case, unless
+// none is masked.  (An instance of its own: the same switch at run time cost
+// the compacted calls 0.2-0.5 us.)
+template <bool kPhilox, bool kLinear, bool kInPlace = false>
 __global__ void __launch_bounds__(kHeadThreads, 1)
 head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
                  const __grid_constant__ CUtensorMap tmap_h,
@@ -1001,27 +1005,20 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
         tma_prefetch_l2_2d(&tmap_w, kb * kBK, (2 * (tk / a.ksplit) + rank) * w_rows);
     }
   }
-  if constexpr (!kLinear) {
+  if constexpr (kInPlace) {
     // (as above: L2 only)
     if (warp == 0 && lane < a.prefetch)
       tma_prefetch_l2_2d(&tmap_w, lane * kBK, (2 * pair + rank) * kBM);
   }
   // Everything below reads what the kernels before it wrote.
   grid_dependency_wait();
-  // Up to kInPlaceRows rows nothing is compacted: all of them go through the
-  // MMAs, which take that many columns in any case, unless none is masked.
-  const bool in_place = !kLinear && a.masked != nullptr;
-  uint32_t flags = 0;
-  int R;
-  if (in_place) {
+  uint32_t flags = 0;                              // kInPlace: the masked rows
+  if constexpr (kInPlace)
     flags = __ballot_sync(0xffffffffu, lane < a.n_flags && a.masked[lane] != 0);
-    R = flags != 0 ? a.n_flags : 0;
-  } else {
-    R = kLinear ? a.linear_rows : *a.n_rows;
-  }
+  const int R = kInPlace ? (flags != 0 ? a.n_flags : 0) : kLinear ? a.linear_rows : *a.n_rows;
   // The layout: hidden rows on the lanes above kPairVocabLanesMax live rows,
   // vocabulary rows on the lanes up to it.
-  const bool rows_mode = kLinear || R > kPairVocabLanesMax;
+  const bool rows_mode = kLinear || (!kInPlace && R > kPairVocabLanesMax);
   // Row groups of 2 x 128 rows (rows mode); each pair takes one group and
   // every per_group-th tile from its first one.
   const int n_groups = R > 2 * kPairRows ? 2 : 1;
@@ -1110,11 +1107,11 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
     for (int i = threadIdx.x - 64; i < n_eff; i += kEpiThreads) {
       // (in place, a row that is not masked reads the first masked row's noise,
       // which costs no traffic; its statistics are not used)
-      rmap[i] = i >= R ? 0 : !in_place ? a.row_map[i] : (flags >> i) & 1u ? i : __ffs(flags) - 1;
+      rmap[i] = i >= R ? 0 : !kInPlace ? a.row_map[i] : (flags >> i) & 1u ? i : __ffs(flags) - 1;
       for (int w = 0; w < 4; ++w) store_stats(wstats(w), i, rowstats_empty());
     }
   }
-  if (in_place && blockIdx.x == 0 && warp == 1) {
+  if (kInPlace && blockIdx.x == 0 && warp == 1) {
     if (lane < a.n_flags) {
       const bool is_live = (flags >> lane) & 1u;
       a.row_map_out[lane] = is_live ? lane : -1;
@@ -1253,7 +1250,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
       const bool row_live = h < R;
       const bool warp_live = __any_sync(0xffffffffu, row_live);
       const int n = !kLinear && row_live ? a.row_map[h] : 0;
-      const bool noisy = !kLinear && a.tau != 0.f && (kPhilox || a.gumbel != nullptr);
+      const bool noisy = kPhilox || (!kLinear && a.tau != 0.f && a.gumbel != nullptr);
       const float* grow = noisy && !kPhilox ? a.gumbel + (size_t)n * a.V : nullptr;
       // kLinear: 32-byte stores where base and row stride allow (each lane
       // writes its own row: 16-byte stores half-fill every sector)
@@ -1372,13 +1369,17 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
                 auto fold = [&](auto full) {
                   constexpr bool kFull = decltype(full)::value;
                   const float mc = fold_sums16<kFull>(st, z, v0, a.V);
-                  if (kPhilox && noisy) {
+                  // (in its first unit a row has new bests often: scoring all
+                  // of it is cheaper there, 512 rows of 512, 8000 ids 51.4 ->
+                  // 45.4 us, 200 rows 34.4 -> 28.3)
+                  if (kPhilox && local > 0) {
                     if (mc != -INFINITY)
                       fold_words16<kFull>(st, z, words, mc, a.tau, inv_tau, v0, a.V);
                   } else {
                     if constexpr (kPhilox) {
 #pragma unroll
-                      for (int j = 0; j < 16; ++j) g[j] = 0.f;
+                      for (int j = 0; j < 16; ++j)
+                        g[j] = sbd_philox::gumbel_of_word(words[j]);
                     }
                     fold_scores16<kFull>(st, z, g, a.tau, v0, a.V);
                   }
@@ -1425,7 +1426,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
       const int quad = warp & 3;
       const StatsRef my_stats = wstats(quad);
       const int sub = (warp - 2) >> 2;          // chunks sub, sub + 2, ... of 16 columns
-      const bool noisy = a.tau != 0.f && (kPhilox || a.gumbel != nullptr);
+      const bool noisy = kPhilox || (a.tau != 0.f && a.gumbel != nullptr);
       const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
       constexpr int kStride = 32;
       const int c_first = 16 * sub;
@@ -1798,7 +1799,7 @@ head_f32_kernel(const float* __restrict__ hidden, const float* __restrict__ w,
   __syncthreads();
   const int v0 = blockIdx.x * kBM;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool noisy = tau != 0.f && (kPhilox || gumbel != nullptr);
+  const bool noisy = kPhilox || (tau != 0.f && gumbel != nullptr);
   const int vq = v0 + 4 * lane;                      // this lane's first id in the reduction
 
   for (int r0 = 0; r0 < R; r0 += kF32Rows) {
@@ -2149,6 +2150,7 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
                        const PhiloxNoise* philox) {
   const int BK = p.B * p.k;
   if (BK == 0) return SBD_OK;
+  if (tau == 0.f) philox = nullptr;                  // no noise
   HeadWs W = head_ws_layout(p, ws);
   sbd_status s;
   cudaError_t e;
@@ -2158,8 +2160,12 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     // CTA pairs from kPairMinRows allocated rows: as many as the device holds
     // at once, the pair tiles need and the workspace has partials for
     // (p.n_ctas), an even number when there may be two row groups.
-    const void* fn_pair = philox ? (const void*)head_pair_kernel<true, false>
-                                 : (const void*)head_pair_kernel<false, false>;
+    const bool few = BK <= kInPlaceRows;
+    const void* fn_pair =
+        philox ? (few ? (const void*)head_pair_kernel<true, false, true>
+                      : (const void*)head_pair_kernel<true, false>)
+               : (few ? (const void*)head_pair_kernel<false, false, true>
+                      : (const void*)head_pair_kernel<false, false>);
     const int pair_tiles = (p.V + 2 * kBM - 1) / (2 * kBM);
     const int n_groups_max = p.rows_alloc > 2 * kPairRows ? 2 : 1;
     int n_pairs = 0;
@@ -2169,7 +2175,7 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
       if (n_pairs > p.n_ctas / 2) n_pairs = p.n_ctas / 2;
       if (n_groups_max == 2) n_pairs &= ~1;
     }
-    const bool in_place = n_pairs > 0 && BK <= kInPlaceRows;
+    const bool in_place = n_pairs > 0 && few;
     if (!in_place) {
       const uint8_t* hid = (const uint8_t*)hidden;
       int bk = BK, rb = p.H * 2;
@@ -2223,7 +2229,7 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     a.off_hi = philox ? (uint32_t)(philox->offset >> 32) : 0u;
     a.row_map = W.row_map;
     a.n_rows = W.n_rows;
-    a.masked = in_place ? masked : nullptr;
+    a.masked = masked;
     a.n_flags = BK;
     a.prefetch = 0;
     if (in_place && (size_t)p.V * p.H * 2 >= kPrefetchMinBytes)

@@ -129,3 +129,17 @@ def test_rows_layout_scores_every_id_that_can_win(sbd, tau, scale):
     e2, t2 = sbd.sbd_head_entropy_sample(hid, w, masked, noise, tau)
     assert torch.equal(t1, t2) and torch.equal(e1, e2)
     assert sbd.sbd_device_error() == 0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("B,k,V", [(2, 16, 700), (5, 16, 700), (16, 16, 600), (1, 4, 100)])
+def test_no_noise_at_tau_zero(sbd, B, k, V, dtype):
+    """tau = 0 takes the kernels without noise, in every layout: the same bits
+    as the buffer call without a buffer, whatever the seed."""
+    import torch
+    d = _case(B, k, V, 128, dtype, seed=k)
+    hid, W = to_dev(d["hidden"], dtype), to_dev(d["w"], dtype)
+    m = torch.from_numpy(d["masked"]).cuda()
+    ent, tok = sbd.sbd_head_entropy_sample_philox(hid, W, m, 3, 4, 0.0)
+    e0, t0 = sbd.sbd_head_entropy_sample(hid, W, m, None, 0.0)
+    assert torch.equal(ent, e0) and torch.equal(tok, t0)
