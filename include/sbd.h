@@ -209,9 +209,10 @@ sbd_status sbd_gumbel_philox(int32_t n_rows, const int32_t* row_ids, int32_t voc
  *
  * y is the fp32 sum over in_features of the bf16 products, rounded to
  * bf16 (round to nearest even).  When a layer has too few output tiles to
- * fill the GPU, the in_features are cut into ranges whose fp32 partials go
- * through the workspace and are summed by a second kernel (the split is
- * chosen per call from the shape).  Above 160 rows the product runs on
+ * fill the GPU, the in_features are cut into ranges whose fp32 partials are
+ * summed in range order: up to 160 rows inside a thread-block cluster where
+ * one of that size fits, else through the workspace by a second kernel (the
+ * split is chosen per call from the shape).  Above 160 rows the product runs on
  * pairs of SMs (2-SM tensor-core MMAs).  All pointers 16-byte aligned,
  * caller-owned.  Asynchronous on `stream`.
  * Supported: dtype bf16, 0 <= rows <= 512, in_features a positive multiple

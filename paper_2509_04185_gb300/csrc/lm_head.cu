@@ -965,7 +965,8 @@ __device__ __forceinline__ void fold_words16(RowStats& st, const float (&z)[16],
 // them go through the MMAs, which take that many columns in any case, unless
 // none is masked.  (An instance of its own: the same switch at run time cost
 // the compacted calls 0.2-0.5 us.)
-template <bool kPhilox, bool kLinear, bool kInPlace = false>
+// kFew: at most kFewRows rows, so never the rows layout.
+template <bool kPhilox, bool kLinear, bool kInPlace = false, bool kFew = kInPlace>
 __global__ void __launch_bounds__(kHeadThreads, 1)
 head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
                  const __grid_constant__ CUtensorMap tmap_h,
@@ -1018,7 +1019,7 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
   const int R = kInPlace ? (flags != 0 ? a.n_flags : 0) : kLinear ? a.linear_rows : *a.n_rows;
   // The layout: hidden rows on the lanes above kPairVocabLanesMax live rows,
   // vocabulary rows on the lanes up to it.
-  const bool rows_mode = kLinear || (!kInPlace && R > kPairVocabLanesMax);
+  const bool rows_mode = kLinear || (!kFew && R > kPairVocabLanesMax);
   // Row groups of 2 x 128 rows (rows mode); each pair takes one group and
   // every per_group-th tile from its first one.
   const int n_groups = R > 2 * kPairRows ? 2 : 1;
@@ -2023,6 +2024,12 @@ constexpr int kPairMinRows = 16;
 // padded N would grow with rows that are not masked.  (Compaction by TMA
 // gather4 loads of the masked rows: 16 rows 158.5 -> 168.8, 64 rows 168 -> 246.)
 constexpr int kInPlaceRows = 32;
+// Rows up to which the compacted call has an instance without the rows layout,
+// whose code had cost the vocabulary layout's in-kernel noise registers: 14 of
+// 60 rows of 1152, 135511 ids 61.7 -> 59.6 us, all 60 76.2 -> 73.9, 36 rows of
+// 1024, 60000 ids 45.8 -> 44.1; 128 rows without noise 41.5 -> 40.9, but 160
+// rows of 4096, 128256 ids 181.2 -> 181.7.
+constexpr int kFewRows = 128;
 // Without the compaction kernel in between, the pair kernel comes up while the
 // kernel before it (attention, in a step) still runs, and its first boxes of W
 // are brought into L2 meanwhile; they are read from there once that kernel is
@@ -2162,10 +2169,12 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
     // (p.n_ctas), an even number when there may be two row groups.
     const bool few = BK <= kInPlaceRows;
     const void* fn_pair =
-        philox ? (few ? (const void*)head_pair_kernel<true, false, true>
-                      : (const void*)head_pair_kernel<true, false>)
-               : (few ? (const void*)head_pair_kernel<false, false, true>
-                      : (const void*)head_pair_kernel<false, false>);
+        philox ? (few               ? (const void*)head_pair_kernel<true, false, true>
+                  : BK <= kFewRows  ? (const void*)head_pair_kernel<true, false, false, true>
+                                    : (const void*)head_pair_kernel<true, false>)
+               : (few               ? (const void*)head_pair_kernel<false, false, true>
+                  : BK <= kFewRows  ? (const void*)head_pair_kernel<false, false, false, true>
+                                    : (const void*)head_pair_kernel<false, false>);
     const int pair_tiles = (p.V + 2 * kBM - 1) / (2 * kBM);
     const int n_groups_max = p.rows_alloc > 2 * kPairRows ? 2 : 1;
     int n_pairs = 0;

@@ -198,12 +198,13 @@ def test_pair_kernel_without_masked_rows(sbd, philox):
 
 
 @pytest.mark.parametrize("which", ["none", "all", "first", "last", "odd"])
-@pytest.mark.parametrize("B,k", [(1, 1), (1, 15), (2, 8), (1, 17), (31, 1), (4, 8), (3, 11)])
+@pytest.mark.parametrize("B,k", [(1, 1), (1, 15), (2, 8), (1, 17), (31, 1), (4, 8), (3, 11),
+                                 (4, 24), (8, 16), (3, 43)])
 def test_bf16_rows_in_place(sbd, B, k, which):
     """Up to 32 rows the pair kernel reads every hidden row where it is: rows
     that are not masked may hold anything (NaN here) without touching the
-    others, and none masked means no work; 33 rows are compacted.  Noise from
-    the buffer and the kernel's own, which must agree bit for bit."""
+    others, and none masked means no work; 33 rows are compacted, and above 128
+    the kernel has both layouts.  Noise from the buffer and the kernel's own, which must agree bit for bit."""
     import torch
     N = B * k
     m = np.zeros(N, dtype=np.uint8)
