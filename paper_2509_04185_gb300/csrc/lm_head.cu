@@ -927,7 +927,10 @@ __device__ __forceinline__ void fold_scores16(RowStats& st, const float (&z)[16]
 // Per call at V = 128256, H = 4096 (bursts), two logarithms a logit against
 // this: 200 rows 227 -> 205 us, 256 rows 225 -> 210, 320 rows 435 -> 385, 512
 // rows 460 -> 380 (the noise buffer: 203, 209, 346, 351); V = 151936, 512
-// rows, under the power cap 480 -> 441-453.  Most of the rest are the generator's
+// rows, under the power cap 480 -> 441-453.  The rule by x_top and a lane's
+// own order took 278 rows of 1280, 31919 ids from 67 to 57 us (98 without the
+// rule when the logits spread 8 times as far; 69 scoring every id), 323 rows
+// of 832, 80096 ids from 111 to 98 (182; 129).  Most of the rest are the generator's
 // rounds.  (Round keys from the host made no difference.)
 template <bool kFull>
 __device__ __forceinline__ void fold_words16(RowStats& st, const float (&z)[16],
@@ -945,14 +948,41 @@ __device__ __forceinline__ void fold_words16(RowStats& st, const float (&z)[16],
 #pragma unroll
   for (int j = 0; j < 16; ++j) x_top = max(x_top, x[j]);
   if (x_top < x_min) return;
+  // A chunk with a new largest logit passes every word; but no noise of the
+  // chunk is above that of x_top, which rules out the ids whose logit is too
+  // far below the best even with it (the same slack).
+  const float g_top = sbd_philox::gumbel_of_word(x_top);
+  const float z_min =
+      st.best - tau * g_top -
+      fmaf(tau, fmaf(fabsf(g_top), 2e-5f, 1e-4f), 1e-6f * (fabsf(st.best) + fabsf(z_max)));
+  // The lanes (rows) find theirs at different j: each takes its own next one,
+  // so that a warp goes round as often as its busiest row has any, not once
+  // for every j that some row has.
+  uint32_t cand = 0u;
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    if (x[j] >= x_min && (kFull || v0 + j < V)) {
-      const float sc = fmaf(tau, sbd_philox::gumbel_of_word(x[j]), z[j]);
-      if (sc > st.best) {
-        st.best = sc;
-        st.idx = v0 + j;
+  for (int j = 0; j < 16; ++j)
+    cand |= x[j] >= x_min && !(z[j] < z_min) && (kFull || v0 + j < V) ? 1u << j : 0u;
+  while (cand != 0u) {
+    const int j = __ffs(cand) - 1;
+    cand &= cand - 1u;
+    uint32_t xs[8];
+    float zs[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      xs[i] = j & 8 ? x[i + 8] : x[i];
+      zs[i] = j & 8 ? z[i + 8] : z[i];
+    }
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+      for (int i = 0; i < w; ++i) {
+        xs[i] = j & w ? xs[i + w] : xs[i];
+        zs[i] = j & w ? zs[i + w] : zs[i];
       }
+    const float sc = fmaf(tau, sbd_philox::gumbel_of_word(xs[0]), zs[0]);
+    if (sc > st.best) {
+      st.best = sc;
+      st.idx = v0 + j;
     }
   }
 }
@@ -1371,8 +1401,9 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
                   constexpr bool kFull = decltype(full)::value;
                   const float mc = fold_sums16<kFull>(st, z, v0, a.V);
                   // (in its first unit a row has new bests often: scoring all
-                  // of it is cheaper there, 512 rows of 512, 8000 ids 51.4 ->
-                  // 45.4 us, 200 rows 34.4 -> 28.3)
+                  // of it is cheaper there: 200 rows of 512, 8000 ids 31.0 ->
+                  // 27.8 us, 512 rows 43.4 -> 40.2; a large vocabulary of 200
+                  // rows 199.8 -> 202.1)
                   if (kPhilox && local > 0) {
                     if (mc != -INFINITY)
                       fold_words16<kFull>(st, z, words, mc, a.tau, inv_tau, v0, a.V);
