@@ -1496,7 +1496,12 @@ static TcKernel attn_tc_kernel_for(const AttnPlan& p) {
 bool attn_use_wide(const AttnPlan& p) {
   if (p.M > kRows / 2) return true;
   if (p.D != 128) return false;
-  if (2ll * p.B * p.Hkv >= 3ll * num_sms()) return p.Lmax <= 3072;
+  // several waves: a few tiles more than one triple cost the wide kernel a
+  // whole second one (32 of 135-159 keys, 5 rows 16.0 paired / 17.4 wide, 64
+  // rows 17.0 / 17.9; of 300-500, 4 rows 22.9 / 23.6, 64 rows 25.7 / 23.7; of
+  // 70-100, one triple, 32 rows 15.4 / 14.0)
+  if (2ll * p.B * p.Hkv >= 3ll * num_sms())
+    return p.Lmax <= 2 * kTileKeys || (p.Lmax > (p.M > 32 ? 256 : 512) && p.Lmax <= 3072);
   return p.Lmax <= (p.M > 32 ? 704ll : 500ll) * p.splits;
 }
 
