@@ -2055,11 +2055,12 @@ constexpr int kPairMinRows = 16;
 // padded N would grow with rows that are not masked.  (Compaction by TMA
 // gather4 loads of the masked rows: 16 rows 158.5 -> 168.8, 64 rows 168 -> 246.)
 constexpr int kInPlaceRows = 32;
-// Rows up to which the compacted call has an instance without the rows layout,
-// whose code had cost the vocabulary layout's in-kernel noise registers: 14 of
-// 60 rows of 1152, 135511 ids 61.7 -> 59.6 us, all 60 76.2 -> 73.9, 36 rows of
-// 1024, 60000 ids 45.8 -> 44.1; 128 rows without noise 41.5 -> 40.9, but 160
-// rows of 4096, 128256 ids 181.2 -> 181.7.
+// Rows up to which the compacted call with in-kernel noise has an instance
+// without the rows layout, whose code had cost the vocabulary layout's noise
+// registers: 14 of 60 rows of 1152, 135511 ids 61.7 -> 59.6 us, all 60 76.2 ->
+// 73.9, 36 rows of 1024, 60000 ids 45.8 -> 44.1; 160 rows of 4096, 128256 ids
+// 198.3 -> 199.7.  (Without noise 128 rows of 1024 41.5 -> 40.9 but 95 of 126
+// rows of 960, 67692 ids 43.1 -> 44.0.)
 constexpr int kFewRows = 128;
 // Without the compaction kernel in between, the pair kernel comes up while the
 // kernel before it (attention, in a step) still runs, and its first boxes of W
@@ -2204,7 +2205,6 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
                   : BK <= kFewRows  ? (const void*)head_pair_kernel<true, false, false, true>
                                     : (const void*)head_pair_kernel<true, false>)
                : (few               ? (const void*)head_pair_kernel<false, false, true>
-                  : BK <= kFewRows  ? (const void*)head_pair_kernel<false, false, false, true>
                                     : (const void*)head_pair_kernel<false, false>);
     const int pair_tiles = (p.V + 2 * kBM - 1) / (2 * kBM);
     const int n_groups_max = p.rows_alloc > 2 * kPairRows ? 2 : 1;
