@@ -199,3 +199,27 @@ def test_reference_passes_between_the_groups(sbd, D, rate):
     d["k_cache"][1, L - 700:] = gen.BF16_NAN
     _check(sbd, w, d, 3, num_splits=1)
     assert sbd.sbd_device_error() == 0
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("G,k,D,n_causal,first_bad", [(1, 3, 64, 2, 1), (4, 4, 128, 4, 2), (4, 8, 128, 3, 3),
+                                                      (2, 32, 64, 16, 16), (4, 32, 128, 17, 9)])
+def test_f32_causal_rows_ignore_later_positions(sbd, G, k, D, n_causal, first_bad, bad):
+    """A causal row sees block keys j <= i only: NaN or infinities in the keys
+    and values of later positions must not reach it, whichever tile and key
+    range holds them."""
+    import torch
+    lens = [0, 1, 58, 63, 64, 200, 513]
+    w = gen.shrink(gen.get_workload("tiny_f32"), batch=len(lens), block_k=k, n_q_heads=G, n_kv_heads=1,
+                   head_dim=D, cache_len=(0, 513 + k))
+    d = _inputs(w, G * k, lens)
+    f = {x: oracle.widen(d[x], "f32") for x in ("q", "k_cache", "v_cache", "k_blk", "v_blk")}
+    ref = oracle.block_attention(f["q"], f["k_cache"], f["v_cache"], d["cache_len"], f["k_blk"],
+                                 f["v_blk"], n_causal=n_causal)
+    for x in ("k_blk", "v_blk"):
+        d[x] = d[x].copy()
+        d[x][:, first_bad:] = bad
+    got = _run(sbd, w, d, n_causal)[0]
+    rows = min(n_causal, first_bad)
+    assert float(np.abs(got[:, :rows] - ref[:, :rows]).max()) <= F32_ATTN_TOL
+    assert sbd.sbd_device_error() == 0
