@@ -1915,7 +1915,7 @@ head_f32_kernel(const float* __restrict__ hidden, const float* __restrict__ w,
       float S = 0.f, T = 0.f;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (vq + j < V) {
+        if (vq + j < V && y[j] != -INFINITY) {       // m may be -inf, too
           const float d = y[j] - m;                  // <= 0
           const float e = exp2f(d);
           S += e;

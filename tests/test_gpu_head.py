@@ -336,3 +336,29 @@ def test_pair_kernel_random_shapes(sbd, case):
             exempt += 1
     assert exempt <= max(1, R // 50)
     assert sbd.sbd_device_error() == 0
+
+
+@pytest.mark.parametrize("R", [3, 12, 20, 32])
+@pytest.mark.parametrize("ids", [(128, 256), (4224, 4352), (4480, 4600)])
+def test_f32_tile_of_minus_infinity_logits(sbd, R, ids):
+    """A vocabulary tile whose logits are all -inf adds nothing: entropy, token
+    and confidence are those of the other ids.  Tiles 33 and 35 of 36 are merged
+    into statistics that their lane already holds."""
+    import torch
+    V, H = 4600, 64
+    g = torch.Generator(device="cuda").manual_seed(R)
+    hid = torch.rand(1, R, H, generator=g, device="cuda") + 0.5
+    w = torch.randn(V, H, generator=g, device="cuda") * 0.3
+    gum = torch.randn(1, R, V, generator=g, device="cuda")
+    m = torch.ones(1, R, dtype=torch.uint8, device="cuda")
+    keep = torch.ones(V, dtype=torch.bool, device="cuda")
+    keep[ids[0]:ids[1]] = False
+    w[~keep] = -float("inf")
+    ent, conf, tok = sbd.sbd_head_entropy_confidence_sample(hid, w, m, gum, 1.0)
+    z = hid[0].double() @ w[keep].double().T
+    p = torch.log_softmax(z, 1)
+    assert float((ent[0] + (p.exp() * p).sum(1)).abs().max()) <= ENTROPY_TOL
+    assert float((conf[0] / p.max(1).values.exp() - 1).abs().max()) <= 1e-4
+    ref = keep.nonzero()[:, 0][(z + gum[0][:, keep].double()).argmax(1)]
+    assert torch.equal(tok[0].long(), ref)
+    assert sbd.sbd_device_error() == 0
