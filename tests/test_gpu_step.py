@@ -100,3 +100,57 @@ def test_llama8b_full_loop(sbd):
 def test_ragged_full_loop(sbd):
     steps, exempt = _loop(sbd, gen.get_workload("ragged_b32_k8"), 0.1)
     assert exempt <= 2
+
+
+@pytest.mark.parametrize("call", ["head", "head_philox", "attention", "causal", "linear"])
+def test_first_cuda_call_of_a_thread(sbd, call):
+    """A host thread whose first use of CUDA is one of the library's calls: the
+    same bits as from the thread that has used it before."""
+    import threading
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(1)
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    st = torch.cuda.current_stream()
+    if call.startswith("head"):
+        hid, w = r(1, 16, 128), r(700, 128)
+        m = torch.ones(1, 16, dtype=torch.uint8, device="cuda")
+        ent, tok = torch.zeros(1, 16, device="cuda"), torch.zeros(1, 16, dtype=torch.int32, device="cuda")
+        ws = torch.empty(1 << 22, dtype=torch.uint8, device="cuda")
+        outs = (ent, tok)
+        if call == "head":
+            go = sbd.prepare_head_entropy_sample(hid, w, m, None, 0.0, ent, tok, ws, stream=st)
+        else:
+            go = sbd.prepare_head_entropy_sample_philox(hid, w, m, 1, 2, 1.0, ent, tok, ws, stream=st)
+    elif call == "linear":
+        y = torch.zeros(5, 300, dtype=torch.bfloat16, device="cuda")
+        outs = (y,)
+        go = sbd.prepare_linear(r(5, 128), r(300, 128), y, stream=st)
+    else:
+        q, kc, vc, kb, vb = r(2, 4, 8, 64), r(2, 90, 2, 64), r(2, 90, 2, 64), r(2, 4, 2, 64), r(2, 4, 2, 64)
+        ln = torch.tensor([80, 13], dtype=torch.int32, device="cuda")
+        out = torch.zeros_like(q)
+        outs = (out, kc, vc)
+        if call == "attention":
+            go = sbd.prepare_block_attention(q, kc, vc, ln, kb, vb, out, stream=st)
+        else:
+            go = lambda: sbd.sbd_block_attention_causal_prefix(q, kc, vc, ln, kb, vb, 2, out, stream=st)
+    go()
+    want = [o.clone() for o in outs]
+    for o in outs[:2 if call.startswith("head") else 1]:
+        o.zero_()
+    torch.cuda.synchronize()
+    errors = []
+
+    def run():
+        try:
+            go()
+        except Exception as e:
+            errors.append(e)
+
+    t = threading.Thread(target=run)
+    t.start()
+    t.join()
+    assert not errors, errors[0]
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(outs, want))
+    assert sbd.sbd_device_error() == 0
