@@ -595,9 +595,8 @@ sbd_status attn_launch(const AttnPlan& p, const void* q, const void* kc, const v
     a.scale_log2 = p.scale_log2;
     const F32Kernel kern = f32_kernel_for(p.D, p.M);
     a.chunks = (p.M + kern.rows - 1) / kern.rows;
-    const cudaError_t e = cudaFuncSetAttribute(
-        kern.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kern.smem);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_f32_kernel)");
+    const sbd_status s = allow_smem(kern.fn, kern.smem, "cudaFuncSetAttribute(attn_f32_kernel)");
+    if (s != SBD_OK) return s;
     void* args[] = {(void*)&a};
     return launch_pdl(kern.fn, dim3(p.splits, p.Hkv * a.chunks, p.B), dim3(kern.threads),
                       kern.smem, st, args, "attn_f32_kernel launch", p.splits);

@@ -1542,8 +1542,8 @@ sbd_status attn_tc_launch(const AttnPlan& p, const CUtensorMap& tk, const CUtens
   const TcKernel kern = attn_tc_kernel_for(p);
   const size_t smem = kern.smem;
   const void* fn = kern.fn;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_tc_kernel)");
+  const sbd_status allowed = allow_smem(fn, smem, "cudaFuncSetAttribute(attn_tc_kernel)");
+  if (allowed != SBD_OK) return allowed;
   // The block keys/values [B, k, Hkv, D] as 4-D tensors (D, Hkv, k, B), read
   // in the cache tiles' boxes (64 columns x 64 rows, 128-byte swizzle): the
   // rows past k are outside the tensor and arrive as zeros.

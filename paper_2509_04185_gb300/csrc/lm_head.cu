@@ -37,7 +37,6 @@
 // kernel's rows layout above.
 #include <math.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "philox.cuh"
@@ -2077,33 +2076,9 @@ constexpr size_t kPrefetchMinBytes = 96u << 20;
 constexpr int kPairRingBytes = 222 * 1024;
 constexpr size_t kPairSmemBytes = 1024 + kPairRingBytes;
 
-// How many clusters of two CTAs of `fn` the current device holds at once
-// (0: none).  Kept per (device, kernel): the call is on every launch's host
-// path.
+// How many CTA pairs of `fn` the current device holds at once (0: none).
 int head_pair_slots(const void* fn) {
-  struct Entry {
-    int dev;
-    const void* fn;
-    int clusters;
-  };
-  static std::mutex mu;
-  static Entry cache[16];
-  static int n_cache = 0;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    for (int i = 0; i < n_cache; ++i)
-      if (cache[i].dev == dev && cache[i].fn == fn) return cache[i].clusters;
-  }
-  const int clusters =
-      sbd::max_active_clusters(fn, dim3(2), dim3(kHeadThreads), kPairSmemBytes, 2);
-  std::lock_guard<std::mutex> lock(mu);
-  if (n_cache < 16) cache[n_cache++] = Entry{dev, fn, clusters};
-  return clusters;
+  return sbd::cluster_slots(fn, kHeadThreads, kPairSmemBytes, 2);
 }
 
 // y = the sum over K ranges of the fp32 partials of sbd_linear, in bf16, each
@@ -2192,7 +2167,6 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
   if (tau == 0.f) philox = nullptr;                  // no noise
   HeadWs W = head_ws_layout(p, ws);
   sbd_status s;
-  cudaError_t e;
   int* err = device_error_word();
   int n_parts = p.n_ctas;   // CTAs that write per-row partials
   if (p.bf16) {
@@ -2314,8 +2288,8 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
       while (cols < (uint32_t)(n_acc_alloc * p.rows_alloc)) cols <<= 1;
       a.tmem_cols = cols;
     }
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(LM head kernel)");
+    s = allow_smem(fn, smem, "cudaFuncSetAttribute(LM head kernel)");
+    if (s != SBD_OK) return s;
     void* args[] = {(void*)&tw, (void*)&th, (void*)&th64, (void*)&th128, (void*)&a};
     s = launch_pdl(fn, dim3(n_parts), dim3(kHeadThreads), smem, st, args,
                    n_pairs > 0 ? "head_pair_kernel launch" : "head_tc_kernel launch",
@@ -2340,8 +2314,8 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
                     (void*)&confidence, (void*)&sk};
     const void* fn =
         philox ? (const void*)head_f32_kernel<true> : (const void*)head_f32_kernel<false>;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32SmemBytes);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(head_f32_kernel)");
+    s = allow_smem(fn, kF32SmemBytes, "cudaFuncSetAttribute(head_f32_kernel)");
+    if (s != SBD_OK) return s;
     s = launch_pdl(fn, dim3(p.n_ctas), dim3(kF32HeadThreads), kF32SmemBytes, st, args, "head_f32_kernel launch");
     if (s != SBD_OK) return s;
   }
@@ -2567,8 +2541,8 @@ sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void
     n_ctas = a.k_cluster || units < slots ? units : slots;
   }
   a.ksplit = ksplit;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(linear kernel)");
+  s = allow_smem(fn, smem, "cudaFuncSetAttribute(linear kernel)");
+  if (s != SBD_OK) return s;
   void* args[] = {(void*)&tw, (void*)&tx, (void*)&tx64, (void*)&tx128, (void*)&a};
   s = launch_pdl(fn, dim3(n_ctas), dim3(kHeadThreads), smem, st, args,
                  T > kPairVocabLanesMax ? "head_pair_kernel (linear) launch" : "head_tc_kernel (linear) launch",

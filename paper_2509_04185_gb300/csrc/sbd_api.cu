@@ -7,6 +7,7 @@
 
 #include <mutex>
 
+#include "launch_cache.h"
 #include "sbd_internal.cuh"
 
 namespace {
@@ -164,20 +165,14 @@ sbd_status launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem, cudaSt
   return SBD_OK;
 }
 
-int max_active_clusters(const void* fn, dim3 grid, dim3 block, size_t smem, int cluster_x) {
-  if (cluster_x > 8 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
+namespace {
+
+// -1 when the driver could not be asked; 0 when it says that the shape cannot
+// be launched as clusters.
+int max_active_clusters(const void* fn, int threads, size_t smem, int cluster_x) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
+  cfg.gridDim = dim3(cluster_x);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -186,40 +181,54 @@ int max_active_clusters(const void* fn, dim3 grid, dim3 block, size_t smem, int 
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  cudaError_t e = cudaSuccess;
+  if (cluster_x > 8)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return n;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
+  if (e == cudaSuccess) return n;
+  cudaGetLastError();
+  return e == cudaErrorInvalidClusterSize || e == cudaErrorInvalidConfiguration ||
+                 e == cudaErrorNotSupported
+             ? 0
+             : -1;
 }
 
-int cluster_slots(const void* fn, int threads, size_t smem, int cluster_x) {
-  struct Entry {
-    int dev;
-    const void* fn;
-    int cluster_x;
-    int clusters;
-  };
-  static std::mutex mu;
-  static Entry kept[64];
-  static int n_kept = 0;
+LaunchCache* launch_cache() {
+  static LaunchCache caches[kMaxDevices];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
-    return 0;
+    return nullptr;
   }
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    for (int i = 0; i < n_kept; ++i)
-      if (kept[i].dev == dev && kept[i].fn == fn && kept[i].cluster_x == cluster_x)
-        return kept[i].clusters;
-  }
-  const int clusters =
-      max_active_clusters(fn, dim3(cluster_x), dim3(threads), smem, cluster_x);
-  std::lock_guard<std::mutex> lock(mu);
-  if (n_kept < 64) kept[n_kept++] = Entry{dev, fn, cluster_x, clusters};
-  return clusters;
+  return dev >= 0 && dev < kMaxDevices ? &caches[dev] : nullptr;
+}
+
+cudaError_t set_smem(LaunchCache& c, const void* fn, size_t smem) {
+  return (cudaError_t)c.allow_smem(fn, smem, [&](size_t most) {
+    return (int)cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  });
+}
+
+}  // namespace
+
+sbd_status allow_smem(const void* fn, size_t smem, const char* what) {
+  LaunchCache* c = launch_cache();
+  if (!c) return fail(SBD_ERR_CUDA, "%s: no current device", what);
+  const cudaError_t e = set_smem(*c, fn, smem);
+  return e == cudaSuccess ? SBD_OK : cuda_fail(e, what);
+}
+
+int cluster_slots(const void* fn, int threads, size_t smem, int cluster_x) {
+  LaunchCache* c = launch_cache();
+  if (!c) return 0;
+  return c->clusters(fn, threads, smem, cluster_x, [&] {
+    if (set_smem(*c, fn, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return -1;
+    }
+    return max_active_clusters(fn, threads, smem, cluster_x);
+  });
 }
 
 }  // namespace sbd

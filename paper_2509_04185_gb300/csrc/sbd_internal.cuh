@@ -99,12 +99,14 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // that size.
 sbd_status launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                       void** args, const char* what, int cluster_x = 1);
-// How many clusters of cluster_x CTAs (with `smem` bytes of dynamic shared
-// memory each) the current device can hold at once; 0 when the shape cannot
-// be launched as clusters.
-int max_active_clusters(const void* fn, dim3 grid, dim3 block, size_t smem, int cluster_x);
-// The same for the current device, kept per (device, kernel, cluster size): for
-// the host path of a launch.
+// Allows `fn` launches with `smem` bytes of dynamic shared memory on the current
+// device; what is allowed already is never taken back (another thread may be
+// about to launch with it).
+sbd_status allow_smem(const void* fn, size_t smem, const char* what);
+// How many clusters of cluster_x CTAs (`threads` threads and `smem` bytes of
+// dynamic shared memory each) the current device can hold at once; 0 when the
+// shape cannot be launched as clusters, or when the driver cannot be asked just
+// now.  Answers are kept: for the host path of a launch.
 int cluster_slots(const void* fn, int threads, size_t smem, int cluster_x);
 
 }  // namespace sbd

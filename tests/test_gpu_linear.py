@@ -101,3 +101,40 @@ def test_random_shapes(sbd, case):
     tol = 2.0 ** -8 * np.abs(ref) + K * 2.0 ** -23 * bound + 1e-6
     assert np.all(np.abs(y - ref) <= tol), (T, K, N, float(np.max(np.abs(y - ref) - tol)))
     assert sbd.sbd_device_error() == 0
+
+
+def test_threads_with_different_row_counts(sbd):
+    """One kernel serves up to 160 rows, with shared memory by the row count:
+    host threads that launch it at the same time, each on its own stream, must
+    not take each other's away."""
+    import threading
+    import torch
+    K, N = 64, 256
+    w = torch.randn(N, K, device="cuda").to(torch.bfloat16)
+    rows = [1, 160, 33, 96]
+    streams = [torch.cuda.Stream() for _ in rows]
+    xs = [torch.randn(r, K, device="cuda").to(torch.bfloat16) for r in rows]
+    ys = [torch.empty(r, N, dtype=torch.bfloat16, device="cuda") for r in rows]
+    calls = [sbd.prepare_linear(x, w, y, stream=s) for x, y, s in zip(xs, ys, streams)]
+    torch.cuda.synchronize()
+    errors = []
+
+    def go(call):
+        try:
+            for _ in range(3000):
+                call()
+        except Exception as e:            # the launch's status
+            errors.append(e)
+
+    ts = [threading.Thread(target=go, args=(c,)) for c in calls]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors[0]
+    for x, y in zip(xs, ys):
+        ref, bound = x.double() @ w.double().T, x.double().abs() @ w.double().abs().T
+        # half a unit in the last place of the output, plus K fp32 additions of the products
+        assert bool(((y.double() - ref).abs() <= 2.0 ** -8 * ref.abs() + K * 2.0 ** -23 * bound + 1e-6).all())
+    assert sbd.sbd_device_error() == 0
