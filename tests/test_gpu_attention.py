@@ -225,3 +225,21 @@ def test_multi_wave_launch_takes_sequences_longest_first(sbd, k, G):
     w = gen.shrink(BF16, batch=40, block_k=k, n_q_heads=8 * G, n_kv_heads=8,
                    cache_len=(0, 512))
     _run_and_compare(sbd, w, seed=k, lens=lens.tolist())
+
+
+@pytest.mark.parametrize("B,k,G,D,lens", [
+    (2, 1, 4, 128, 4096), (1, 4, 4, 128, 2000), (3, 16, 4, 128, 700), (2, 1, 4, 64, 4096), (4, 16, 4, 64, 700)])
+def test_paired_kernel_repeats_bit_for_bit(sbd, B, k, G, D, lens):
+    """One to nine pairs a split, in turn from 40 lengths: the last reference and
+    the last product pass between the two groups of softmax warps, and whichever
+    comes first, the bits are the same."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(lens + k)
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    q, kb, vb = r(B, k, 8 * G, D) * 2, r(B, k, 8, D), r(B, k, 8, D)
+    kc, vc = r(B, lens, 8, D), r(B, lens, 8, D)
+    for n in range(lens - 64 * 39, lens + 1, 64) if lens >= 2496 else range(0, lens + 1, lens // 39):
+        ln = torch.full((B,), max(0, n), dtype=torch.int32, device="cuda")
+        outs = [sbd.sbd_block_attention(q, kc, vc, ln, kb, vb) for _ in range(6)]
+        assert all(torch.equal(outs[0], o) for o in outs[1:]), n
+    assert sbd.sbd_device_error() == 0
