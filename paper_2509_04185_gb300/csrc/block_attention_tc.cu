@@ -324,19 +324,20 @@ __device__ __forceinline__ void merge_rows(const TcArgs& a, int b, int hkv, uint
   }
 }
 
-// (Head dimension 64 takes its rows one at a time: the other forms inlined
-// there cost that kernel's main loop 1.5 %; a call instead of inlining, 1-2 us
-// of every launch.)
-template <int D>
+// Few instances: every one inlined costs every launch, also those that take
+// another.  Against one for each of 2, 4, 8 and more splits, as many rows as fill
+// the registers: 128 rows, batch 1, 100 keys of a capacity of 1024 12.0 -> 11.1
+// us, 4 rows, batch 1, 100 of 8192 7.17 -> 7.07; 128 rows, batch 8, 4096 keys in
+// clusters of 2 32.6 either way.  With <16, 1> alone 64 rows of the last took 31.7
+// for 30.7.  (A call instead of inlining: 1-2 us of every launch.)
+template <int D, bool kWide>
 __device__ __forceinline__ void cluster_merge(const TcArgs& a, int b, int hkv, uint32_t cpart_s,
                                               int sw, int lane) {
   cluster_sync_all();
   if (sw >= 0 && sw < kSoftWarps) {
     const int rank = (int)cluster_ctarank();
-    if (D == 64) merge_rows<D, 16, 1>(a, b, hkv, cpart_s, rank, sw, lane);
-    else if (a.splits <= 2) merge_rows<D, 2, 8>(a, b, hkv, cpart_s, rank, sw, lane);
-    else if (a.splits <= 4) merge_rows<D, 4, 4>(a, b, hkv, cpart_s, rank, sw, lane);
-    else if (a.splits <= 8) merge_rows<D, 8, 2>(a, b, hkv, cpart_s, rank, sw, lane);
+    if (D == 128 && kWide && a.splits <= 2) merge_rows<D, 2, 4>(a, b, hkv, cpart_s, rank, sw, lane);
+    else if (D == 128 && a.splits <= 4) merge_rows<D, 4, 2>(a, b, hkv, cpart_s, rank, sw, lane);
     else merge_rows<D, 16, 1>(a, b, hkv, cpart_s, rank, sw, lane);
   }
   cluster_sync_all();
@@ -965,7 +966,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     tc_fence_after();
     tc_dealloc(tmem, kTmemCols);
   }
-  if (a.cluster) cluster_merge<D>(a, b, hkv, kv_s + 65536u, warp - 2, lane);
+  if (a.cluster) cluster_merge<D, false>(a, b, hkv, kv_s + 65536u, warp - 2, lane);
 }
 
 // ------------------------------------------------------------ wide row tiles
@@ -1468,7 +1469,7 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_k,
     tc_fence_after();
     tc_dealloc(tmem, kTmemCols);
   }
-  if (a.cluster) cluster_merge<D>(a, b, hkv, k_s, warp - 3, lane);
+  if (a.cluster) cluster_merge<D, true>(a, b, hkv, k_s, warp - 3, lane);
 }
 
 }  // namespace
