@@ -1506,24 +1506,36 @@ static TcKernel attn_tc_kernel_for(const AttnPlan& p) {
                   kWideThreads, attn_wide_smem_bytes(p.D)};
 }
 
-// Above 64 packed rows only attn_wide_kernel serves.  Up to 64, at head
-// dimension 128, it is the faster one where a CTA has few keys (its triples
-// come through in fewer steps: 16 rows x 4 heads, batch 1, 500 / 1000 / 4096
-// keys, i.e. up to 341 a CTA, 9.9 / 10.5 / 11.7 us paired, 9.0 / 9.6 / 11.1
-// wide; batch 4, 2000 keys, 500 a CTA, 14.6 / 13.6; with few rows the line
-// lies lower: batch 2, 4096 keys, 512 a CTA, 64 rows 15.4 / 15.2 but 4 rows
-// 13.0 / 13.6), and where short sequences take several waves (its end is
-// shorter: 64 of 500-2000 keys 80.9 / 77.9; 32 of 4096 94.9 / 97.0).
+// Above 64 packed rows only attn_wide_kernel serves, at head dimension 64 and up
+// to 64 rows only attn_tc_kernel.  Elsewhere (measured over batch 1-64, 32 query
+// heads over 8, lengths 64-8000 at capacities of once and 4 times the length,
+// paired / wide):
+//   up to 128 keys    a cache's two tiles and the block's are one triple: batch
+//                     64, 100 keys, 16 rows 30.0 / 28.7 us, 32 rows 32.8 / 30.0;
+//                     batch 4, 16 rows 6.6 / 6.6;
+//   above 32 rows     wide as far as a CTA has few keys, then both load at the
+//                     memory's rate and the paired kernel's pipeline is finer:
+//                     batch 1, 1000 keys 9.6 / 9.2, batch 4, 2000 (500 a CTA)
+//                     14.2 / 13.3, batch 12, 4096 a CTA 43.0 / 46.3; in several
+//                     waves batch 32, 300 keys 21.5 / 19.7, batch 64, 2000 100.5 /
+//                     96.4, batch 32, 4096 81.9 / 82.3;
+//   17 to 32 rows     wide in several waves of middling lengths: batch 64, 300 of
+//                     1200 keys 39.8 / 37.1, but batch 32, 200 of 200 16.4 / 17.1;
+//   up to 16 rows     the same from three waves on, batch 64, 100 of 1024, 16 rows
+//                     32.0 / 29.9; else paired: its steps are finer (a triple for
+//                     4 tiles is two), batch 16, 159 keys, 4 rows 7.5 / 8.5, batch
+//                     2, 159 of 636, 16 rows 7.5 / 8.2, batch 32, 1000, 4 rows
+//                     31.3 / 32.4.
+// The capacity stands for the lengths, which the host does not know; with
+// lengths a quarter of it the choice is still the faster one or within 5 %.
 bool attn_use_wide(const AttnPlan& p) {
   if (p.M > kRows / 2) return true;
   if (p.D != 128) return false;
-  // several waves: a few tiles more than one triple cost the wide kernel a
-  // whole second one (32 of 135-159 keys, 5 rows 16.0 paired / 17.4 wide, 64
-  // rows 17.0 / 17.9; of 300-500, 4 rows 22.9 / 23.6, 64 rows 25.7 / 23.7; of
-  // 70-100, one triple, 32 rows 15.4 / 14.0)
-  if (2ll * p.B * p.Hkv >= 3ll * num_sms())
-    return p.Lmax <= 2 * kTileKeys || (p.Lmax > (p.M > 32 ? 256 : 512) && p.Lmax <= 3072);
-  return p.Lmax <= (p.M > 32 ? 704ll : 500ll) * p.splits;
+  if (p.Lmax <= 2 * kTileKeys) return true;
+  const long long jobs = (long long)p.B * p.Hkv, sms = num_sms();
+  if (2 * jobs >= 3 * sms)                     // several waves
+    return (p.M > 16 || jobs >= 3 * sms) && p.Lmax > (p.M > 32 ? 0 : 512) && p.Lmax <= 3072;
+  return p.M > 32 && p.Lmax <= 704ll * p.splits;
 }
 
 bool attn_tc_cluster_ok(const AttnPlan& p, int splits) {

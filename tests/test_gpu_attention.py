@@ -243,3 +243,36 @@ def test_paired_kernel_repeats_bit_for_bit(sbd, B, k, G, D, lens):
         outs = [sbd.sbd_block_attention(q, kc, vc, ln, kb, vb) for _ in range(6)]
         assert all(torch.equal(outs[0], o) for o in outs[1:]), n
     assert sbd.sbd_device_error() == 0
+
+
+@pytest.mark.parametrize("G,k", [(1, 4), (4, 4), (3, 8), (4, 16)])
+@pytest.mark.parametrize("B,line", [(12, 128), (28, 128), (28, 512), (28, 3072), (29, 512), (57, 512), (57, 3072), (12, 704)])
+def test_both_sides_of_the_kernel_choice(sbd, B, line, G, k):
+    """Capacities at and one past the lines between the paired and the wide kernel:
+    one triple (128 keys), middling and long caches in several waves of CTAs (28 or
+    29 sequences of 8 heads on 148-152 SMs) and in three (57), one range of 704 keys
+    a CTA (12).  Lengths from nothing to the capacity, at the tiles' edges."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(line + B)
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    D, H = 128, 8
+    for cap in (line, line + 1):
+        q, kb, vb = r(B, k, H * G, D) * 2, r(B, k, H, D), r(B, k, H, D)
+        kc, vc = r(B, cap, H, D), r(B, cap, H, D)
+        pool = [0, 1, 63, 64, 65, 127, 128, 129, 191, 192, 193, 257, 320, min(cap, 700)]
+        lens = [min(cap, pool[b % len(pool)]) for b in range(B)]
+        lens[B // 2] = cap
+        for b, n in enumerate(lens):
+            kc[b, n:] = float("nan")
+            vc[b, n:] = float("nan")
+        out = sbd.sbd_block_attention(q, kc, vc, torch.tensor(lens, dtype=torch.int32, device="cuda"), kb, vb)
+        for b, n in enumerate(lens):
+            kk = torch.cat([kc[b, :n], kb[b]]).float().repeat_interleave(G, 1)
+            vv = torch.cat([vc[b, :n], vb[b]]).float().repeat_interleave(G, 1)
+            p = torch.softmax(torch.einsum("ihd,nhd->hin", q[b].float(), kk) / D ** 0.5, -1)
+            ref, size = torch.einsum("hin,nhd->ihd", p, vv), torch.einsum("hin,nhd->ihd", p, vv.abs())
+            # the probabilities and the output are rounded to 8 bits (half a unit: 2^-8 of
+            # each), the sums are in 32
+            tol = 2.0 ** -8 * (size + ref.abs()) + 1e-3
+            assert bool(((out[b].float() - ref).abs() <= tol).all()), (cap, b, n)
+    assert sbd.sbd_device_error() == 0
