@@ -71,6 +71,18 @@ def test_split_and_unit_edges(sbd, T, K, N):
     assert sbd.sbd_device_error() == 0
 
 
+@pytest.mark.parametrize("T,K,N", [
+    # rows of outputs, or of fp32 partials, that start on 16 bytes but not on 32, on 8 and on 2
+    (161, 512, 1000), (300, 512, 1000), (512, 512, 1000), (161, 1024, 100), (257, 1024, 100), (200, 2048, 1004),
+    (512, 64, 24), (161, 2048, 1002), (384, 2048, 1001),
+    # up to 160 rows: 16, 8, 4 and 2 K ranges through the workspace, fewer and more outputs than are summed
+    # four at a time, and a count that four does not divide
+    (1, 4096, 1024), (160, 4096, 1024), (128, 8192, 2048), (64, 2048, 2048), (33, 2048, 2049), (100, 8192, 2050),
+    (160, 4096, 28672), (96, 4096, 2048), (5, 64 * 12, 20001)])
+def test_store_widths_and_range_sums(sbd, T, K, N):
+    test_split_and_unit_edges(sbd, T, K, N)
+
+
 def test_out_of_range_rows_are_not_written(sbd):
     import torch
     rng = np.random.default_rng(1)
