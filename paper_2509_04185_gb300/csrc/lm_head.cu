@@ -67,10 +67,14 @@ constexpr int kEpiWarps = 8;
 // spills registers.
 constexpr int kGAhead = 3;
 constexpr int kEpiThreads = 32 * kEpiWarps;
-// kLinear: K ranges of a cluster at most, and stages per range at least for
-// the longer stages (so that whole stages split evenly).
+// kLinear: K ranges of a cluster at most.
 constexpr int kMaxRanges = 8;
-constexpr int kRangeStages = 4;
+// kLinear: whether K ranges of whole stages are about as long as each other.
+// (Stages of one 64-column box instead, for ranges alike to the box: 1024 x 1024
+// at 1 to 160 rows 5.8-8.25 us, with stages of 4 boxes 5.3-8.0.)
+__host__ __device__ constexpr bool even_ranges(int stages, int ranges) {
+  return stages % ranges == 0 || stages >= 4 * ranges;
+}
 constexpr int kHeadThreads = 64 + kEpiThreads;   // warp 0 TMA, warp 1 MMA, then the epilogue
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -523,7 +527,7 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
   int boxes = kMaxBoxes;
   while (boxes > 1 &&
          ((a.H / kBK) % boxes != 0 || !fits(boxes, boxes > 2 ? 3 : 2) ||
-          (ksplit > 1 && (a.H / kBK) / boxes < kRangeStages * ksplit)))
+          !even_ranges(a.H / kBK / boxes, ksplit)))
     boxes >>= 1;
   const int stage_bytes = boxes * (kABytes + b_box);     // [A boxes | B boxes]
   int stages = ring_bytes / stage_bytes;
@@ -2095,37 +2099,56 @@ int head_pair_slots(const void* fn) {
 }
 
 // y = the sum over K ranges of the fp32 partials of sbd_linear, in bf16, each
-// element in range order.  kVec: 4 outputs a thread (16-byte reads, every
-// range of the group of 4 in flight), for T N a multiple of 4, where every
-// range starts on 16 bytes; otherwise one output a thread.  (One output a
-// thread took 10 us for 2 ranges of 512 x 4096, ~4 with 4; their
-// 21 MB, out of L2, are 3.1 us of HBM time.)
-template <bool kVec>
+// element in range order, with every range of an element requested at once.
+// kVec: 4 outputs a thread, for T N a multiple of 4, where every range starts on
+// 16 bytes, and from kReduceVec outputs on; fewer leave the threads too few: 1 to
+// 64 rows of 1024 in 16 ranges, 4096 columns deep, 6.9-8.5 us with 4 outputs a
+// thread, 6.4-7.8 with one; 128 rows of 4096 in 4 ranges 13.5 / 15.0.  (4 ranges
+// requested at a time: those 1 to 64 rows 8.2-9.6 us.)
+constexpr long long kReduceVec = 192 << 10;
+template <int kRanges, bool kVec>
 __global__ void __launch_bounds__(256)
-linear_reduce_kernel(const float* __restrict__ part, int ksplit, long long tn,
-                     __nv_bfloat16* __restrict__ y) {
+linear_reduce_kernel(const float* __restrict__ part, long long tn, __nv_bfloat16* __restrict__ y) {
   grid_dependency_wait();
   grid_dependents_launch();
   const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * (kVec ? 4 : 1);
   if (i >= tn) return;
   if constexpr (kVec) {
+    float4 v[kRanges];
+#pragma unroll
+    for (int ks = 0; ks < kRanges; ++ks)
+      v[ks] = *reinterpret_cast<const float4*>(part + (size_t)ks * tn + i);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-    for (int ks = 0; ks < ksplit; ++ks) {
-      const float4 v = *reinterpret_cast<const float4*>(part + (size_t)ks * tn + i);
-      acc.x += v.x;
-      acc.y += v.y;
-      acc.z += v.z;
-      acc.w += v.w;
+#pragma unroll
+    for (int ks = 0; ks < kRanges; ++ks) {
+      acc.x += v[ks].x;
+      acc.y += v[ks].y;
+      acc.z += v[ks].z;
+      acc.w += v[ks].w;
     }
     uint2 w;
     w.x = pack_bf16x2(acc.x, acc.y);
     w.y = pack_bf16x2(acc.z, acc.w);
     *reinterpret_cast<uint2*>(y + i) = w;
   } else {
+    float v[kRanges];
+#pragma unroll
+    for (int ks = 0; ks < kRanges; ++ks) v[ks] = part[(size_t)ks * tn + i];
     float acc = 0.f;
-    for (int ks = 0; ks < ksplit; ++ks) acc += part[(size_t)ks * tn + i];
+#pragma unroll
+    for (int ks = 0; ks < kRanges; ++ks) acc += v[ks];
     y[i] = __float2bfloat16_rn(acc);
+  }
+}
+
+// The instance for a power of two of K ranges, 2 to 16.
+template <bool kVec>
+const void* linear_reduce_for(int ranges) {
+  switch (ranges) {
+    case 2: return (const void*)linear_reduce_kernel<2, kVec>;
+    case 4: return (const void*)linear_reduce_kernel<4, kVec>;
+    case 8: return (const void*)linear_reduce_kernel<8, kVec>;
+    default: return (const void*)linear_reduce_kernel<16, kVec>;
   }
 }
 
@@ -2429,14 +2452,20 @@ static PairSplit pair_linear_split(int T, int K, int N, int n_pairs) {
 }
 
 // K ranges of the single-CTA linear kernel's tiles as clusters, all running at
-// once (1: no split): as many as the SMs hold, each at least 4 column blocks.
-// The ranges then add up through distributed shared memory, with no fp32
-// partials in HBM and no second kernel: 4096 -> 6144 columns at 128 rows
-// 21.2 -> 18.0 us, at 160 rows 25.8 -> 20.8; at 16 rows within 0.3 us.
-static int linear_cluster_ranges(const void* fn, size_t smem, int T, int K, int n_tiles) {
+// once (1: through the workspace): as many as the SMs hold, each at least 4
+// column blocks, of even length.  The ranges then add up through distributed
+// shared memory, with no fp32 partials in HBM and no second kernel: 4096 -> 4096
+// columns at 128 rows 13.5 -> 12.6 us, at 160 rows 16.3 -> 14.6, 4096 -> 6144 17.9
+// -> 17.2, 22.3 -> 20.9; 1024 -> 1024 at 16 rows 6.1 -> 5.7.  Where clusters cannot
+// be as many CTAs as the split through the workspace (8 a tile at most, and what
+// fits in the GPU's parts) that one is taken: 2048 -> 2048 at 1 row 7.4 us in
+// clusters of 7, 6.3 in 8 ranges; 8192 -> 2048 at 64 rows 13.1 / 11.8.
+static int linear_cluster_ranges(const void* fn, size_t smem, int T, int K, int n_tiles, int ksplit) {
   if (T > kPairVocabLanesMax) return 1;   // T x 128 partials fit the ring
-  for (int ks = kMaxRanges; ks > 1; --ks)
-    if (n_tiles * ks <= num_sms() && K / kBK >= 4 * ks &&
+  int boxes = kMaxBoxes;
+  while ((K / kBK) % boxes != 0) boxes >>= 1;
+  for (int ks = kMaxRanges; ks > 1 && ks >= ksplit; --ks)
+    if (n_tiles * ks <= num_sms() && K / kBK >= 4 * ks && even_ranges(K / kBK / boxes, ks) &&
         cluster_slots(fn, kHeadThreads, smem, ks) >= n_tiles)
       return ks;
   return 1;
@@ -2544,7 +2573,7 @@ sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void
     while (cols < (uint32_t)(n_acc_alloc * rows_alloc)) cols <<= 1;
     a.tmem_cols = cols;
     const int slots = num_sms();
-    const int in_cluster = linear_cluster_ranges(fn, smem, T, K, a.n_tiles);
+    const int in_cluster = linear_cluster_ranges(fn, smem, T, K, a.n_tiles, ksplit);
     if (in_cluster > 1) {
       ksplit = in_cluster;
       a.k_cluster = 1;
@@ -2564,11 +2593,10 @@ sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void
   const float* part = (const float*)ws;
   long long tn = (long long)T * N;
   __nv_bfloat16* yb = (__nv_bfloat16*)y;
-  int ks = ksplit;
-  void* rargs[] = {(void*)&part, (void*)&ks, (void*)&tn, (void*)&yb};
-  const bool vec = tn % 4 == 0;
+  void* rargs[] = {(void*)&part, (void*)&tn, (void*)&yb};
+  const bool vec = tn % 4 == 0 && tn >= kReduceVec;
   const long long threads = vec ? tn / 4 : tn;
-  return launch_pdl(vec ? (const void*)linear_reduce_kernel<true> : (const void*)linear_reduce_kernel<false>,
+  return launch_pdl(vec ? linear_reduce_for<true>(ksplit) : linear_reduce_for<false>(ksplit),
                     dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, rargs,
                     "linear_reduce_kernel launch");
 }
