@@ -864,6 +864,7 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
 // rows, against 2070 MHz and ~450 W for head_tc_kernel) and lost to it.
 constexpr int kPairRows = 128;                 // hidden rows of one CTA per unit (M / 2)
 constexpr int kPairVocabLanesMax = 160;        // live rows up to which the vocabulary layout runs
+constexpr int kPrefetchAtOnce = 4;             // in place: boxes of W brought into L2 unasked
 
 // One 16-column chunk of a row's logits z (vocabulary ids v0 .. v0 + 15, valid
 // below V; kFull: all of them are) folded into the running maximum and sums;
@@ -1040,9 +1041,19 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
     }
   }
   if constexpr (kInPlace) {
-    // (as above: L2 only)
-    if (warp == 0 && lane < a.prefetch)
+    // (as above: L2 only.)  With no row masked W is not read: the greater part
+    // follows once a flag is seen, on a warp that has nothing else to do yet.  The
+    // flags may still change before the wait below; here they only decide about
+    // the prefetch, and the load stays out of L1.
+    if (warp == 0 && lane < min(a.prefetch, kPrefetchAtOnce))
       tma_prefetch_l2_2d(&tmap_w, lane * kBK, (2 * pair + rank) * kBM);
+    if (warp == 2 && a.prefetch > kPrefetchAtOnce) {
+      uint32_t flag = 0;
+      if (lane < a.n_flags)
+        asm volatile("ld.relaxed.gpu.global.u8 %0, [%1];" : "=r"(flag) : "l"(a.masked + lane));
+      if (__any_sync(0xffffffffu, flag != 0) && lane >= kPrefetchAtOnce && lane < a.prefetch)
+        tma_prefetch_l2_2d(&tmap_w, lane * kBK, (2 * pair + rank) * kBM);
+    }
   }
   // Everything below reads what the kernels before it wrote.
   grid_dependency_wait();
@@ -2084,8 +2095,10 @@ constexpr int kFewRows = 128;
 // done.  16 boxes: 32000 ids of 2048 29.3 -> 27.7 us (8 boxes 28.4; 32 27.8),
 // 50304 of 1024 24.0 -> 23.2, 151936 of 4096 182.8 -> 180.7, 128256 158.3 ->
 // 156.1.  A W that stays in L2 from call to call only loses (82 MB: 24.8 ->
-// 25.7 us; 41 MB 17.2 -> 18.0), and W below about this size does.  (With no row
-// masked they are read for nothing: 5.6 -> 6.4 us.)
+// 25.7 us; 41 MB 17.2 -> 18.0), and W below about this size does.  With no row
+// masked they would be read for nothing, so all but kPrefetchAtOnce wait for a
+// flag: 16 rows, none masked, of 2048, 32003 ids 6.5 us with all of them at once,
+// 5.5 so, 5.2 with none at once, which costs the other calls (27.9 us) 0.5.
 constexpr int kPrefetchBoxes = 16;
 constexpr size_t kPrefetchMinBytes = 96u << 20;
 // its ring: what is left of the 227 KB of a CTA next to its static shared

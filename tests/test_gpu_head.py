@@ -362,3 +362,31 @@ def test_f32_tile_of_minus_infinity_logits(sbd, R, ids):
     ref = keep.nonzero()[:, 0][(z + gum[0][:, keep].double()).argmax(1)]
     assert torch.equal(tok[0].long(), ref)
     assert sbd.sbd_device_error() == 0
+
+
+@pytest.mark.parametrize("B,k", [(1, 1), (1, 16), (4, 8)])
+def test_bf16_early_reads_of_a_large_weight(sbd, B, k):
+    """A weight large enough that its first part is brought into L2 before the
+    kernel's wait, most of it only when a row is seen masked: nothing masked, all,
+    one, and flags that a kernel just before the call sets or clears."""
+    import torch
+    V, H = 25003, 2048
+    g = torch.Generator(device="cuda").manual_seed(B * k)
+    hid = torch.randn(B, k, H, generator=g, device="cuda").to(torch.bfloat16)
+    w = (torch.randn(V, H, generator=g, device="cuda") * 0.02).to(torch.bfloat16)
+    z = hid.view(-1, H).double() @ w.double().T
+    p = torch.log_softmax(z, 1)
+    ref_e, ref_t = -(p.exp() * p).sum(1), z.argmax(1)
+    m = torch.zeros(B, k, dtype=torch.uint8, device="cuda")
+    ws = torch.empty(64 << 20, dtype=torch.uint8, device="cuda")
+    one = torch.zeros(B * k, dtype=torch.uint8, device="cuda")
+    one[-1] = 1
+    for flags in (torch.zeros_like(one), torch.ones_like(one), torch.zeros_like(one), one, 1 - one, torch.ones_like(one)):
+        m.view(-1).copy_(flags)
+        ent, tok = sbd.sbd_head_entropy_sample(hid, w, m, None, 0.0, workspace=ws)
+        on = flags.bool()
+        e, t = ent.view(-1), tok.view(-1)
+        assert bool(torch.isinf(e[~on]).all()) and bool((t[~on] == -1).all())
+        assert not on.any() or float((e - ref_e)[on].abs().max()) <= ENTROPY_TOL
+        assert torch.equal(t[on].long(), ref_t[on])
+    assert sbd.sbd_device_error() == 0
