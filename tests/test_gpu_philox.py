@@ -111,15 +111,22 @@ def test_fresh_offsets_give_fresh_samples(sbd):
 
 @pytest.mark.parametrize("tau", [1e-35, 1e-3, 1.0, 40.0])
 @pytest.mark.parametrize("scale", [0.0, 1e-3, 1.0, 300.0])
-def test_rows_layout_scores_every_id_that_can_win(sbd, tau, scale):
-    """Above 160 rows the in-kernel noise is turned into a score only where its
-    random word can beat the best so far: the winner must be that of scoring
-    every id (the same noise from a buffer), bit for bit, for logits that are
-    all equal, small, ordinary and huge, weak and strong noise, and a
-    vocabulary that ends inside a 16-id chunk."""
+@pytest.mark.parametrize("B,k,H,V,later", [(12, 16, 128, 9001, False),      # one unit a pair, nearly
+                                           (12, 16, 64, 76009, True),       # one row group, four units a pair
+                                           (18, 16, 64, 40009, True)])      # two row groups, likewise
+def test_rows_layout_scores_every_id_that_can_win(sbd, tau, scale, B, k, H, V, later):
+    """Above 160 rows the in-kernel noise of a row's second unit and later ones is
+    turned into a score only where its random word can beat the best so far: the
+    winner must be that of scoring every id (the same noise from a buffer), bit
+    for bit, for logits that are all equal, small, ordinary and huge, weak and
+    strong noise, and a vocabulary that ends inside a 16-id chunk."""
     import torch
+    # a pair of SMs takes 256 ids a unit, and there is one pair for two SMs and
+    # row group at most: the ids of all first units
+    pairs = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    first = 256 * (pairs // (2 if B * k > 256 else 1))
+    assert not later or 2 * first < V
     g = torch.Generator(device="cuda").manual_seed(3)
-    B, k, H, V = 12, 16, 128, 9001
     hid = (torch.randn(B, k, H, generator=g, device="cuda") * scale).to(torch.bfloat16)
     w = torch.randn(V, H, generator=g, device="cuda").to(torch.bfloat16)
     masked = torch.ones(B, k, dtype=torch.uint8, device="cuda")
@@ -128,6 +135,8 @@ def test_rows_layout_scores_every_id_that_can_win(sbd, tau, scale):
     e1, t1 = sbd.sbd_head_entropy_sample_philox(hid, w, masked, 77, 11, tau)
     e2, t2 = sbd.sbd_head_entropy_sample(hid, w, masked, noise, tau)
     assert torch.equal(t1, t2) and torch.equal(e1, e2)
+    # and winners do lie there (equal logits without noise that counts: id 0 wins)
+    assert not later or (scale == 0.0 and tau < 1e-30) or int((t1 >= first).sum()) > B * k // 4
     assert sbd.sbd_device_error() == 0
 
 
