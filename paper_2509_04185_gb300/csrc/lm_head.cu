@@ -70,10 +70,16 @@ constexpr int kEpiThreads = 32 * kEpiWarps;
 // kLinear: K ranges of a cluster at most.
 constexpr int kMaxRanges = 8;
 // kLinear: whether K ranges of whole stages are about as long as each other.
-// (Stages of one 64-column box instead, for ranges alike to the box: 1024 x 1024
-// at 1 to 160 rows 5.8-8.25 us, with stages of 4 boxes 5.3-8.0.)
-__host__ __device__ constexpr bool even_ranges(int stages, int ranges) {
+constexpr bool even_ranges(int stages, int ranges) {
   return stages % ranges == 0 || stages >= 4 * ranges;
+}
+// Boxes of a stage at most for H columns in `ranges` K ranges: whole stages, and
+// even ranges of them.  (Single boxes, for ranges alike to the box: 1024 -> 1024 at
+// 1 to 160 rows 5.8-8.25 us, with stages of 4 boxes 5.3-8.0.)
+int stage_boxes(int H, int ranges) {
+  int b = kMaxBoxes;
+  while (b > 1 && ((H / kBK) % b != 0 || !even_ranges(H / kBK / b, ranges))) b >>= 1;
+  return b;
 }
 constexpr int kHeadThreads = 64 + kEpiThreads;   // warp 0 TMA, warp 1 MMA, then the epilogue
 constexpr float kLog2e = 1.4426950408889634f;
@@ -436,6 +442,7 @@ struct HeadArgs {
   int ksplit;           // kLinear: K ranges per output tile (1: y written directly)
   int w_rows;           // kLinear, pairs: W rows of a unit per CTA (a multiple of 16 up to 128)
   int k_cluster;        // kLinear: the ranges of a tile form one cluster and add up there
+  int boxes;            // head_tc_kernel: 64-column boxes of a stage at most
   float* part_y;        // kLinear, ksplit > 1: fp32 partials [ksplit][linear_rows][V]
   // kInPlace: the flags of all n_flags rows, and what the compaction kernel
   // writes otherwise
@@ -523,12 +530,13 @@ head_tc_kernel(const __grid_constant__ CUtensorMap tmap_w,
   // and the (tile, range) units are spread over the CTAs
   const int ksplit = kLinear ? a.ksplit : 1;
   const int n_units = a.n_tiles * ksplit;
-  auto fits = [&](int bx, int n_st) { return ring_bytes / (bx * (kABytes + b_box)) >= n_st; };
-  int boxes = kMaxBoxes;
-  while (boxes > 1 &&
-         ((a.H / kBK) % boxes != 0 || !fits(boxes, boxes > 2 ? 3 : 2) ||
-          !even_ranges(a.H / kBK / boxes, ksplit)))
-    boxes >>= 1;
+  // (a.boxes divides the columns.  Every division here is on the way to the first
+  // load: with the ranges' part of this choice in the kernel, and fits() a
+  // division, an 8B layer's four GEMMs took 86.6 us at 16 rows, 86.1 so, those of
+  // a layer of 1024 and 2816 columns 26.8 and 24.6)
+  auto fits = [&](int bx, int n_st) { return ring_bytes >= n_st * bx * (kABytes + b_box); };
+  int boxes = kMaxBoxes;         // (4, 2 or 1, as the compiler sees: the loops over it are unrolled)
+  while (boxes > 1 && (boxes > a.boxes || !fits(boxes, boxes > 2 ? 3 : 2))) boxes >>= 1;
   const int stage_bytes = boxes * (kABytes + b_box);     // [A boxes | B boxes]
   int stages = ring_bytes / stage_bytes;
   if (stages > kMaxStages) stages = kMaxStages;
@@ -2337,6 +2345,7 @@ sbd_status head_launch(const HeadPlan& p, const void* hidden, const void* w,
       while (cols < (uint32_t)(n_acc_alloc * p.rows_alloc)) cols <<= 1;
       a.tmem_cols = cols;
     }
+    a.boxes = stage_boxes(p.H, 1);
     s = allow_smem(fn, smem, "cudaFuncSetAttribute(LM head kernel)");
     if (s != SBD_OK) return s;
     void* args[] = {(void*)&tw, (void*)&th, (void*)&th64, (void*)&th128, (void*)&a};
@@ -2475,10 +2484,11 @@ static PairSplit pair_linear_split(int T, int K, int N, int n_pairs) {
 // clusters of 7, 6.3 in 8 ranges; 8192 -> 2048 at 64 rows 13.1 / 11.8.
 static int linear_cluster_ranges(const void* fn, size_t smem, int T, int K, int n_tiles, int ksplit) {
   if (T > kPairVocabLanesMax) return 1;   // T x 128 partials fit the ring
-  int boxes = kMaxBoxes;
-  while ((K / kBK) % boxes != 0) boxes >>= 1;
-  for (int ks = kMaxRanges; ks > 1 && ks >= ksplit; --ks)
-    if (n_tiles * ks <= num_sms() && K / kBK >= 4 * ks && even_ranges(K / kBK / boxes, ks) &&
+  const int pairs = (K / kBK) % 2 == 0 ? 2 : 1;         // boxes of a stage: two, where even
+  // (through the workspace the units go to the SMs in rounds: so many at a time)
+  const int sms = num_sms(), units = n_tiles * ksplit, in_ws = units / ((units + sms - 1) / sms);
+  for (int ks = kMaxRanges; ks > 1 && n_tiles * ks >= in_ws; --ks)
+    if (n_tiles * ks <= sms && K / kBK >= 4 * ks && even_ranges(K / kBK / pairs, ks) &&
         cluster_slots(fn, kHeadThreads, smem, ks) >= n_tiles)
       return ks;
   return 1;
@@ -2596,6 +2606,7 @@ sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void
     n_ctas = a.k_cluster || units < slots ? units : slots;
   }
   a.ksplit = ksplit;
+  a.boxes = stage_boxes(K, ksplit);
   s = allow_smem(fn, smem, "cudaFuncSetAttribute(linear kernel)");
   if (s != SBD_OK) return s;
   void* args[] = {(void*)&tw, (void*)&tx, (void*)&tx64, (void*)&tx128, (void*)&a};
