@@ -2485,8 +2485,13 @@ static PairSplit pair_linear_split(int T, int K, int N, int n_pairs) {
 static int linear_cluster_ranges(const void* fn, size_t smem, int T, int K, int n_tiles, int ksplit) {
   if (T > kPairVocabLanesMax) return 1;   // T x 128 partials fit the ring
   const int pairs = (K / kBK) % 2 == 0 ? 2 : 1;         // boxes of a stage: two, where even
-  // (through the workspace the units go to the SMs in rounds: so many at a time)
-  const int sms = num_sms(), units = n_tiles * ksplit, in_ws = units / ((units + sms - 1) / sms);
+  // (Through the workspace the units go to the SMs in rounds, so many at a time;
+  // three quarters of that in clusters, one launch with the next one's W on its way,
+  // are as good: the GEMMs of a layer of 3072 and 8192 columns, 48 rows 57.4 -> 55.4 us,
+  // of an 8B layer, 16 rows 86.2 -> 84.8, though 4096 -> 6144 by itself 12.8 -> 13.3 at
+  // 1 row.  With a single round not: 8192 -> 2048 at 1 row, 128 CTAs 9.5, 112 11.3.)
+  const int sms = num_sms(), units = n_tiles * ksplit, rounds = (units + sms - 1) / sms;
+  const int in_ws = rounds == 1 ? units : 3 * units / (4 * rounds);
   for (int ks = kMaxRanges; ks > 1 && n_tiles * ks >= in_ws; --ks)
     if (n_tiles * ks <= sms && K / kBK >= 4 * ks && even_ranges(K / kBK / pairs, ks) &&
         cluster_slots(fn, kHeadThreads, smem, ks) >= n_tiles)
