@@ -137,13 +137,14 @@ attn_combine_kernel(const float* __restrict__ part_o, const float* __restrict__ 
 // workspace is needed.
 // Bound: the FMAs of a full tile are 2 us of an SM (32 rows x 64 keys x 128
 // dimensions, twice); a tile measured 5.2 us with one CTA on the SM, the rest
-// being latencies between the phases that a second CTA covers in part.  With
-// 4 warps of 8 rows in place of 8 of 4: 30.3 against 28.6 us at the shape below.
+// being latencies between the phases, which a second CTA covers in part, and
+// reads of shared memory (S: 12 cycles of its port for 8 of FMAs; PV: 20 for
+// 16).  With 4 warps of 8 rows in place of 8 of 4: 6 % slower at the shape below.
 // The form before (one CTA per query row and head, each walking all keys,
 // uncoalesced) took 717 us at B = 2, k = 8, 32/8 heads of 128, 511-2048
 // cached keys, and 37 us at 4/2 heads of 64, k = 4, 128 keys (the smallest
-// configuration); this one takes 28.6 and 4.6 us (graph replays; the FMAs of
-// the first are 4.2 us of the whole chip, its bytes 3.1 us of HBM).
+// configuration); this one takes 27-29 us by the lengths drawn, and 4.7 (the FMAs
+// of the first are 4.2 us of the whole chip, its bytes 3.1 us of HBM).
 constexpr int kF32Keys = 64;                 // keys per tile
 constexpr int kF32Granule = 16;              // key ranges are multiples of this
 

@@ -32,9 +32,10 @@
 //
 // Both tcgen05 kernels also serve sbd_linear (y = x W^T, a template
 // switch): the same main loop over all rows of x, an epilogue that stores
-// the outputs (or, with K split over CTAs, fp32 partials that
-// linear_reduce_kernel sums); head_tc_kernel up to 160 rows, the pair
-// kernel's rows layout above.
+// the outputs; head_tc_kernel up to 160 rows, the pair kernel's rows layout
+// above.  With K split over CTAs the fp32 partials of a tile add up inside a
+// thread-block cluster (up to 160 rows, where clusters are as good a split), or
+// go through the workspace to linear_reduce_kernel.
 #include <math.h>
 
 #include <type_traits>
@@ -1626,12 +1627,13 @@ head_pair_kernel(const __grid_constant__ CUtensorMap tmap_w,
 //
 // Bound: W's bytes up to ~16 rows, the FMAs above (128 per SM and cycle).
 // The form before read both operands of every scalar FMA from shared memory
-// with one stage and one thread per vocabulary row.  Per call with the
-// compaction and the merge, V = 32003, H = 2048 (262 MB of W: 39 us; 32 rows
-// of FMAs: 52 us, 63 with the 251 tiles on 152 SMs): 18-30 rows 714-926 us
-// before, 132 now; 16 rows 75, 8 rows 51.  Shared memory returns 128 bytes a
-// cycle to registers, broadcasts included: with 8 rows x 4 ids a lane (12
-// reads for 128 FMAs) the reads bound it (32 rows 148 us).
+// with one stage and one thread per vocabulary row.  Per call with the merge,
+// V = 32003, H = 2048 (262 MB of W: 39 us; 32 rows of FMAs: 52 us, 63 with the
+// 251 tiles on 152 SMs): 1-8 rows 397-528 us before, 53 now; 9-16 rows 548-677
+// and 72; 17-24 rows 700-835 and 105; 25-32 rows 853-985 and 128.5.  Shared
+// memory returns 128 bytes a cycle to registers, broadcasts included: with 8
+// rows x 4 ids a lane (12 reads for 128 FMAs) the reads bound it (32 rows 12 %
+// slower).
 constexpr int kF32HeadWarps = 8;
 constexpr int kF32HeadThreads = 32 * kF32HeadWarps;
 constexpr int kF32Cols = 32;
@@ -1832,7 +1834,7 @@ head_f32_kernel(const float* __restrict__ hidden, const float* __restrict__ w,
   // flags), the first one writes them out for the merge, and the unmasked
   // rows' results; the hidden rows are read where they are.  A kernel of its own
   // that did this and copied the rows, as for bf16, cost a launch: 1-3 rows of
-  // hidden 256, 512 ids 8.8 -> 7.6 us, 32 rows of 2048, 32003 ids 132 -> 128.5.
+  // hidden 256, 512 ids 8.8 -> 7.6 us, 32 rows of 2048, 32003 ids 3.5 us.
   __shared__ int rows_sh[kF32MaxRows], count_sh[kF32MaxRows / 32];
   grid_dependency_wait();
   for (int i0 = 0; i0 < kF32MaxRows; i0 += kF32HeadThreads) {
@@ -2439,10 +2441,10 @@ int linear_ksplit(int T, int K, int N) {
 // shortest modelled time.  A 64-column block of a unit takes as long as its
 // rows' fill of shared memory (107 GB/s an SM, measured in the main loop at
 // 512 rows) or its four 2-SM MMAs (44 ns up to N = 128, 65 at N = 256), and no
-// less than 0.235 us (measured at 32 and 64 W rows); units go to the pairs of their row group in rounds.  Fewer W rows a unit fill a
-// round better (512 x 6144, 38 pairs a group: 24 units of 256 ids, 32 of
-// 192); K ranges shorten the units but write fp32 partials that a second
-// kernel reads back.  At most linear_max_split ranges (what the workspace
+// less than 0.235 us (measured at 32 and 64 W rows); units go to the pairs of
+// their row group in rounds.  Fewer W rows a unit fill a round better (512 x
+// 6144, 38 pairs a group: 24 units of 256 ids, 32 of 192); K ranges shorten the
+// units but write fp32 partials that a second kernel reads back.  At most linear_max_split ranges (what the workspace
 // holds).  Against 128 W rows throughout (an 8B layer's four GEMMs): 256 rows
 // 126.0 -> 120.4 us, 512 rows 165.3 -> 162.5 in bursts.
 struct PairSplit {

@@ -72,8 +72,10 @@ struct PhiloxNoise {
   uint64_t seed, offset;
 };
 // y[T, N] = x[T, K] W[N, K]^T, bf16 in and out, fp32 accumulation; T <= 512.
-// At few rows K is split over CTAs (linear_ksplit ranges), with fp32 partials
-// in the workspace (linear_workspace_bytes) summed by a second kernel.
+// With few output tiles K is split over CTAs: in clusters that add their fp32
+// partials up (up to 160 rows, chosen in linear_launch), or in linear_ksplit
+// ranges with the partials in the workspace (linear_workspace_bytes) and a
+// second kernel.
 int linear_ksplit(int T, int K, int N);
 size_t linear_workspace_bytes(int T, int K, int N);
 sbd_status linear_launch(int T, int K, int N, const void* x, const void* w, void* y, void* ws,
@@ -94,7 +96,9 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Launch with programmatic dependent launch allowed: the kernel may be
 // scheduled while its predecessor on the stream finishes; every library
-// kernel calls griddepcontrol.wait before it touches global memory.
+// kernel calls griddepcontrol.wait before it uses or writes global memory.
+// (Before it some bring weights into L2, which stays coherent, and the LM head
+// looks at the flags to decide whether to.)
 // cluster_x > 1: CTAs of consecutive blockIdx.x form thread-block clusters of
 // that size.
 sbd_status launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -165,11 +165,11 @@ def test_f32_split_and_tile_edges(sbd, G, k, D, n_causal):
 @pytest.mark.parametrize("splits", [1, 2, 3, 6])
 @pytest.mark.parametrize("G,k,D", [(1, 2, 128), (4, 4, 128), (3, 11, 128), (4, 16, 128), (4, 16, 64), (1, 5, 64)])
 def test_bf16_both_kernels_up_to_64_rows(sbd, G, k, D, splits, n_causal):
-    """Up to 64 packed rows: capacities on both sides of the line between the
-    wide and the paired kernel (500 or 704 keys a split at head dimension
-    128), lengths that end a pair, a tile and the hand-over between the
-    paired kernel's two groups (1 to 5 pairs, odd and even, the last of one
-    tile or two)."""
+    """Up to 64 packed rows: capacities around 500 keys a split, and above 32 rows
+    on both sides of the line between the wide and the paired kernel (704 keys a
+    split at head dimension 128), lengths that end a pair, a tile and the
+    hand-over between the paired kernel's two groups (1 to 5 pairs, odd and
+    even, the last of one tile or two)."""
     lens = [0, 1, 63, 64, 65, 128, 191, 192, 256, 257, 320, 449, 576]
     line = (704 if G * k > 32 else 500) * splits
     for cap in (line, line + 1):
