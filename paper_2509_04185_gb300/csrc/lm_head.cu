@@ -2444,9 +2444,10 @@ int linear_ksplit(int T, int K, int N) {
 // less than 0.235 us (measured at 32 and 64 W rows); units go to the pairs of
 // their row group in rounds.  Fewer W rows a unit fill a round better (512 x
 // 6144, 38 pairs a group: 24 units of 256 ids, 32 of 192); K ranges shorten the
-// units but write fp32 partials that a second kernel reads back.  At most linear_max_split ranges (what the workspace
-// holds).  Against 128 W rows throughout (an 8B layer's four GEMMs): 256 rows
-// 126.0 -> 120.4 us, 512 rows 165.3 -> 162.5 in bursts.
+// units but write fp32 partials that a second kernel reads back.  At most
+// linear_max_split ranges (what the workspace holds).  Against 128 W rows
+// throughout (an 8B layer's four GEMMs): 256 rows 126.0 -> 120.4 us, 512 rows
+// 165.3 -> 162.5 in bursts.
 struct PairSplit {
   int w_rows, ksplit;
 };
